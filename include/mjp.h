@@ -110,9 +110,11 @@ extern "C" {
                                    of FP32 two-state models whose observation groups have at most two members (one
                                    CTA of MJP_OPT_THREADS / 32 <= 8 warps per theta; automatic when 0) and for
                                    expv_series of birth-death models (automatic thread count), none with a forced
-                                   cluster size, else the shared-memory kernel), 1 = shared-memory
+                                   cluster size; else, without a forced thread count or cluster size, the kernel with
+                                   registers and a shared-memory tile (groups of at most two members), else the
+                                   shared-memory kernel), 1 = shared-memory
                                    kernel, 2 = register-resident kernel (MJP_ERR_UNSUPPORTED where it does not
-                                   apply; other models' expv_series always runs the shared-memory kernel).  Also a batch option
+                                   apply; other models' expv_series runs the shared-memory kernel).  Also a batch option
                                    (expv_batch_set_option): 0 = the register-resident birth-death kernel wherever every
                                    instance fits it (N_j <= 8 x 6,720 states FP32, 8 x 3,360 FP64), 1 = shared-memory
                                    kernel, 2 = register-resident kernel */
@@ -131,9 +133,10 @@ extern "C" {
                                    the register-resident two-state log-likelihood chain (the hand-over of observation
                                    chunks between its chain and reducer warps) and the register-resident
                                    mRNA/protein log-likelihood chain (the hand-over of the block rows that cross
-                                   from one CTA of a cluster to the next, every jump).  A wait that runs out stops
-                                   the CSR and two-state chains; the mRNA/protein chain stops waiting and runs on to
-                                   its end with invalid values.  rate_model_check then returns
+                                   from one CTA of a cluster to the next, every jump) and the register/tile kernel
+                                   on clusters (the same, every few jumps).  A wait that runs out stops
+                                   the CSR and two-state chains; the others stop waiting and run on to
+                                   their end with invalid values.  rate_model_check then returns
                                    MJP_ERR_DEVICE_TIMEOUT */
 
 typedef struct mjp_model mjp_model;

@@ -11,6 +11,7 @@
 
 #include "host_util.h"
 #include "internal.cuh"
+#include "tile_plan.h"
 
 using namespace mjp;
 
@@ -191,6 +192,19 @@ double omega_bound(const mjp_model* m, const double* th) {
       return 1.1 * (th[0] + (th[1] + th[2]) * (double)(m->M - 1) + (th[3] + th[5]) * (double)(m->P / 2 - 1) + th[4]);
     default: return 0.0;
   }
+}
+
+// How many of the times' windows (about 16 sqrt(x) jumps each) hold a jump on
+// average, at the model's own theta; steers launch shapes only.
+double window_overlap(const mjp_model* m, const double* times, int nt) {
+  const double om = omega_bound(m, m->theta.data());
+  double sum = 0.0, top = 1.0;
+  for (int i = 0; i < nt; ++i) {
+    const double x = om * times[i];
+    sum += 16.0 * std::sqrt(x) + 3.0;
+    top = std::max(top, x);
+  }
+  return std::min((double)nt, sum / (top + 6.0 * std::sqrt(top)));
 }
 
 // Make room in the weight arena for B instances at the given times: windows
@@ -740,10 +754,14 @@ int expv_series(mjp_model* m, const void* rho0, const double* times, int ntimes,
   if (m->chain == 2 && m->kind == MJP_BD1D && !use_reg1)
     return fail(MJP_ERR_UNSUPPORTED, "the register-resident expv chain needs a birth-death model without "
                                      "a forced thread count that fits 8 CTAs");
+  // Other models at the automatic shape: the register/tile chain, where it fits.
+  TilePlan xp = {};
+  const bool use_tile = !use_reg1 && m->chain == 0 && m->cluster == 0 && m->threads == 0 && m->kcap <= (1 << 30) - 1 &&
+                        tile_plan(m->kind, m->precision, false, m->M, m->P, nt, 0, 0, 1, window_overlap(m, st.data(), nt), &xp);
   int C = 0, T = 0;
   int64_t slab = 0;
   int rc = 0;
-  if (!use_reg1 && (rc = stencil_config(m, 0, nt, 0, 0, &C, &T, &slab))) return rc;
+  if (!use_reg1 && !use_tile && (rc = stencil_config(m, 0, nt, 0, 0, &C, &T, &slab))) return rc;
   if ((rc = ensure_status(m))) return rc;
   if ((rc = m->d_times.ensure(sizeof(double) * nt))) return rc;
   if ((rc = m->d_orig.ensure(sizeof(int32_t) * nt))) return rc;
@@ -774,8 +792,9 @@ int expv_series(mjp_model* m, const void* rho0, const double* times, int ntimes,
   cp.orig = m->d_orig.as<int32_t>(); cp.win = pp.win; cp.info = pp.info; cp.rho0 = rho0;
   cp.out = out; cp.out_stride = 0; cp.comp = m->d_comp.as<float>(); cp.comp_stride = 0;
   cp.renorm = (m->precision == MJP_FP32) ? m->renorm : 0;
-  cp.slab = slab; cp.status = pp.status;
+  cp.slab = slab; cp.status = pp.status; cp.wait_limit = m->wait_limit;
   if (use_reg1) MJP_CUDA(launch_chain_reg1d(m->precision, cp, rp1, s));
+  else if (use_tile) MJP_CUDA(launch_chain_tile(m->kind, m->precision, false, cp, xp, s));
   else MJP_CUDA(launch_chain_stencil(m->kind, m->precision, 0, cp, C, T, s));
   if ((rc = mark(m, 2, s))) return rc;
 
@@ -1054,7 +1073,13 @@ int loglik(mjp_model* m, const mjp_obs* obs, const double* theta, int B, double*
                                      "CTAs, at the automatic thread count or 256, or an FP32 two-state model whose "
                                      "groups have at most two members and that fits one CTA");
   int rc = 0;
-  if (!use_reg && !use_ts && (rc = stencil_config(m, 1, nt, obs->G, nmem_list, &C, &T, &slab))) return rc;
+  // Other models at the automatic shape: the register/tile chain, where it fits.
+  TilePlan xp = {};
+  const bool use_tile = !use_reg && !use_ts && m->chain == 0 && m->cluster == 0 && m->threads == 0 &&
+                        m->kcap <= (1 << 30) - 1 &&
+                        tile_plan(m->kind, m->precision, true, m->M, m->P, nt, obs->G, obs->maxmem, B,
+                                  window_overlap(m, obs->times.data(), nt), &xp);
+  if (!use_reg && !use_ts && !use_tile && (rc = stencil_config(m, 1, nt, obs->G, nmem_list, &C, &T, &slab))) return rc;
   if ((rc = ensure_status(m))) return rc;
   if ((rc = m->d_win.ensure(sizeof(Win) * (size_t)nt * B))) return rc;
   if ((rc = m->d_info.ensure(sizeof(JobInfo) * (size_t)B))) return rc;
@@ -1100,6 +1125,7 @@ int loglik(mjp_model* m, const mjp_obs* obs, const double* theta, int B, double*
   cp.job_map = ordered ? m->d_jmap.as<int32_t>() : nullptr;
   if (use_reg) MJP_CUDA(launch_chain_reg2d(cp, rp, s));
   else if (use_ts) MJP_CUDA(launch_chain_regts(cp, tp, s));
+  else if (use_tile) MJP_CUDA(launch_chain_tile(m->kind, m->precision, true, cp, xp, s));
   else MJP_CUDA(launch_chain_stencil(m->kind, m->precision, 1, cp, C, T, s));
   if ((rc = mark(m, 2, s))) return rc;
   if (where == MJP_PTR_HOST) {

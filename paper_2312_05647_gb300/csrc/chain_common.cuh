@@ -101,6 +101,51 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
+// Hand-over of states that cross a CTA boundary of a cluster.  A sending
+// thread writes its 16 bytes into the neighbour CTA's shared memory with
+// st.async, which counts them on that CTA's hand-over mbarrier (one per
+// direction and parity of the hand-over); the receiving threads wait for the
+// phase they need, and one of them re-arms the barrier with the bytes it
+// expects two hand-overs later.  Addresses are 32-bit shared-memory addresses (mapa gives the
+// neighbour's copy of a variable).
+__device__ __forceinline__ unsigned cluster_addr(unsigned local, int rank) {
+  unsigned r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void hbar_init(unsigned a) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(a) : "memory");
+}
+__device__ __forceinline__ void hbar_arm(unsigned a, unsigned bytes) {
+  asm volatile("{ .reg .b64 st; mbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1; }" ::"r"(a), "r"(bytes)
+               : "memory");
+}
+// At most `polls` tests of the phase of parity ph (none when polls is 0):
+// false when the phase has not completed by then.  The test acquires at
+// cluster scope: the bytes it orders were written by another CTA.
+__device__ __forceinline__ bool hbar_wait(unsigned a, unsigned ph, long long polls) {
+  for (long long i = 0; i < polls; ++i) {
+    unsigned ok;
+    asm volatile(
+        "{ .reg .pred p; mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
+        : "=r"(ok) : "r"(a), "r"(ph) : "memory");
+    if (ok) return true;
+    if (i >= 16) __nanosleep(32);
+  }
+  return false;
+}
+__device__ __forceinline__ void st_async16(unsigned raddr, float2 a, float2 b, unsigned rbar) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(
+                   raddr),
+               "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "r"(rbar)
+               : "memory");
+}
+__device__ __forceinline__ void st_async16(unsigned raddr, double2 a, unsigned rbar) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f64 [%0], {%1, %2}, [%3];" ::"r"(raddr),
+               "d"(a.x), "d"(a.y), "r"(rbar)
+               : "memory");
+}
+
 // Scaled rates (rate / Omega) of one instance in the chain type.
 template <typename T>
 struct Coef {
@@ -260,6 +305,35 @@ __device__ __forceinline__ float mrna_defect(const MrnaCol& col, float gp, int p
   const float dpf = __fmul_rn(gp, fp);
   const float row = dpf >= col.e0 ? __fsub_rn(__fsub_rn(e, dpf), col.e0) : __fsub_rn(__fsub_rn(e, col.e0), dpf);
   return __fadd_rn(col.eps, row);
+}
+
+
+// The same by model kind, for the state in tile row `row`, column `col` of the
+// kernels that hold every kind (stencil.cu, stencil_tile.cuh); the
+// autoregulatory model forms it in FP64 from the FP32 coefficients of its update.
+template <int KIND, typename T>
+__device__ __forceinline__ float exit_defect(const Coef<T>& co, int row, int col, int M, int P) {
+  if (KIND == MJP_BD1D) return bd_defect(co, col, M);
+  if (KIND == MJP_MRNA_PROT2D) return mrna_defect(mrna_col(co, col, M), (float)co.d, row);
+  if (KIND == MJP_TWOSTATE) return ts_defect(co, row, col, M);
+  const float fm = (float)col;
+  // Autoregulatory network, tile row 2 q + sigma (Pm = P / 2 protein counts).
+  const int q = row >> 1, Pm = P / 2;
+  const float fq = (float)q;
+  const bool qtop = q + 1 >= Pm;
+  const float a_gm = __fmul_rn((float)co.c, fm);                // gamma_R m (to m-1)
+  const float a_tx = col + 1 < M ? (float)co.a : 0.0f;          // beta_R (to m+1, active)
+  const float tr = qtop ? 0.0f : __fmul_rn((float)co.b, fm);    // beta_P m (to q+1)
+  const float pd = __fmul_rn((float)co.d, fq);                  // gamma_P q (to q-1)
+  const float decay = __fadd_rn(pd, a_gm);
+  if ((row & 1) == 0) {
+    const float bind = __fmul_rn((float)co.f, fq);              // lambda_ina q (to q-1, inactive)
+    const float e = __fadd_rn(__fadd_rn(__fadd_rn(decay, a_tx), tr), bind);
+    return (float)(((((double)e - (double)a_tx) - (double)a_gm) - (double)tr) - (double)pd - (double)bind);
+  }
+  const float unb = qtop ? 0.0f : (float)co.e;                  // lambda_act (to q+1, active)
+  const float e = __fadd_rn(__fadd_rn(decay, tr), unb);
+  return (float)(((((double)e - (double)a_gm) - (double)tr) - (double)pd) - (double)unb);
 }
 
 }  // namespace

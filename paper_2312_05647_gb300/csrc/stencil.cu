@@ -138,37 +138,6 @@ __host__ __device__ inline Smem smem_layout(size_t elt, int tile, int nt, int G,
   return s;
 }
 
-// Exit defect of the state in tile row `row`, column `col` for the compensated
-// FP32 chain (see chain_common.cuh): the exit coefficient the update applies
-// minus the sum of the outflow coefficients its neighbours apply.  Birth-death
-// and mRNA/protein use the shared forms (their chains also run in the
-// register-resident kernels); the two-state and autoregulatory models form it
-// in FP64 from the FP32 coefficients of the update below.
-template <int KIND, typename T>
-__device__ float exit_defect(const Coef<T>& co, int row, int col, int M, int P) {
-  if (KIND == MJP_BD1D) return bd_defect(co, col, M);
-  if (KIND == MJP_MRNA_PROT2D) return mrna_defect(mrna_col(co, col, M), (float)co.d, row);
-  if (KIND == MJP_TWOSTATE) return ts_defect(co, row, col, M);
-  const float fm = (float)col;
-  // Autoregulatory network, tile row 2 q + sigma (Pm = P / 2 protein counts).
-  const int q = row >> 1, Pm = P / 2;
-  const float fq = (float)q;
-  const bool qtop = q + 1 >= Pm;
-  const float a_gm = __fmul_rn((float)co.c, fm);                // gamma_R m (to m-1)
-  const float a_tx = col + 1 < M ? (float)co.a : 0.0f;          // beta_R (to m+1, active)
-  const float tr = qtop ? 0.0f : __fmul_rn((float)co.b, fm);    // beta_P m (to q+1)
-  const float pd = __fmul_rn((float)co.d, fq);                  // gamma_P q (to q-1)
-  const float decay = __fadd_rn(pd, a_gm);
-  if ((row & 1) == 0) {
-    const float bind = __fmul_rn((float)co.f, fq);              // lambda_ina q (to q-1, inactive)
-    const float e = __fadd_rn(__fadd_rn(__fadd_rn(decay, a_tx), tr), bind);
-    return (float)(((((double)e - (double)a_tx) - (double)a_gm) - (double)tr) - (double)pd - (double)bind);
-  }
-  const float unb = qtop ? 0.0f : (float)co.e;                  // lambda_act (to q+1, active)
-  const float e = __fadd_rn(__fadd_rn(decay, tr), unb);
-  return (float)(((((double)e - (double)a_gm) - (double)tr) - (double)pd) - (double)unb);
-}
-
 template <typename T, int KIND, bool LL>
 __global__ void __launch_bounds__(1024, 1) chain_kernel(ChainParams p) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -585,9 +554,11 @@ __global__ void __launch_bounds__(1024, 1) chain_kernel(ChainParams p) {
               y = comp_finish(cur, t, l);
               *lp = l;
             } else {
-              const T2 t1 = v_fma(c_l, left, v_mul(c_dg, cur));
-              const T2 t2 = v_fma(c_sw, v_make(cur.y, cur.x), v_mul(c_r, right));
-              y = v_add(t1, t2);
+              // In the order of stencil_tile.cuh.
+              y = v_mul(c_dg, cur);
+              y.x = f_fma(co.a, left.x, y.x);
+              y = v_fma(c_r, right, y);
+              y = v_fma(c_sw, v_make(cur.y, cur.x), y);
             }
           } else if (KIND == MJP_AUTOREG) {
             // Pair = (active, inactive) at protein count q: transcription from

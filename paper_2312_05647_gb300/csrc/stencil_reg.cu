@@ -207,45 +207,6 @@ __device__ __forceinline__ void tmem_st4(unsigned taddr, float2 a, float2 b) {
 }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
-// Hand-over of the block rows that cross a CTA boundary.  A sending thread
-// writes its 16 bytes into the neighbour CTA's row array with st.async, which
-// counts them on that CTA's hand-over mbarrier (one per direction and jump
-// parity); the receiving threads wait for the phase of the jump they need,
-// and the first of them re-arms the barrier with the bytes it expects two
-// jumps later.  Addresses are 32-bit shared-memory addresses (mapa gives the
-// neighbour's copy of a variable).
-__device__ __forceinline__ unsigned cluster_addr(unsigned local, int rank) {
-  unsigned r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local), "r"(rank));
-  return r;
-}
-__device__ __forceinline__ void hbar_init(unsigned a) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(a) : "memory");
-}
-__device__ __forceinline__ void hbar_arm(unsigned a, unsigned bytes) {
-  asm volatile("{ .reg .b64 st; mbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1; }" ::"r"(a), "r"(bytes)
-               : "memory");
-}
-// At most `polls` tests of the phase of parity ph (none when polls is 0):
-// false when the phase has not completed by then.  The test acquires at
-// cluster scope: the bytes it orders were written by another CTA.
-__device__ __forceinline__ bool hbar_wait(unsigned a, unsigned ph, long long polls) {
-  for (long long i = 0; i < polls; ++i) {
-    unsigned ok;
-    asm volatile(
-        "{ .reg .pred p; mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
-        : "=r"(ok) : "r"(a), "r"(ph) : "memory");
-    if (ok) return true;
-    if (i >= 16) __nanosleep(32);
-  }
-  return false;
-}
-__device__ __forceinline__ void st_async16(unsigned raddr, float2 a, float2 b, unsigned rbar) {
-  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(
-                   raddr),
-               "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "r"(rbar)
-               : "memory");
-}
 // Plain store into a neighbour CTA (ordered by a later cluster barrier).
 __device__ __forceinline__ void st_cluster16(unsigned raddr, float2 a, float2 b) {
   asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(raddr), "f"(a.x), "f"(a.y), "f"(b.x),

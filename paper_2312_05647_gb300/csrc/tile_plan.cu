@@ -1,0 +1,148 @@
+// tile_plan.cu -- choice of the launch shape of the register/tile jump chain
+// (stencil_tile.cuh) and its dispatch.
+#include <algorithm>
+#include <cmath>
+
+#include "internal.cuh"
+#include "tile_plan.h"
+
+namespace mjp {
+
+namespace {
+
+constexpr int kSms = 152;
+
+// Pairs per thread that are instantiated (tile_ll32.cu and its like).
+const int* runs_of(int kind, int precision, bool ll, bool cl) {
+  static const int bd32[] = {1, 2, 4, 8, 0}, ar32[] = {1, 2, 4, 6, 10, 0}, r124[] = {1, 2, 4, 0};
+  static const int r123[] = {1, 2, 3, 0}, r14[] = {1, 4, 0}, r24[] = {2, 4, 0}, r12[] = {1, 2, 0}, r23456[] = {2, 3, 4, 5, 6, 0};
+  static const int none[] = {0};
+  const bool row = kind == MJP_BD1D || kind == MJP_TWOSTATE;
+  if (ll) {
+    if (precision == MJP_FP32 && kind == MJP_MRNA_PROT2D) return none;  // stencil_reg.cu
+    if (cl) return row ? r14 : r24;
+    if (precision == MJP_FP64) return r124;
+    return kind == MJP_BD1D ? bd32 : kind == MJP_TWOSTATE ? r124 : ar32;
+  }
+  if (kind == MJP_BD1D) return none;  // stencil_reg1d.cu
+  if (precision == MJP_FP64) return cl && row ? r12 : r123;
+  return !cl ? r124 : row ? r12 : r23456;
+}
+
+}  // namespace
+
+// The shape with the least estimated time, in cycles per jump.  FP32: a base
+// of about 250 (row kinds) or 450 (grid kinds) cycles of latency and 15 per
+// pair and warp, 4 more per overlapping window (fitted on the 200 x 200
+// mRNA/protein box: 3 to 6 pairs per thread on 13 and 19 warps, 1,530 to 1,920
+// cycles without hand-overs, within 2%).  FP64: every operation holds a
+// scheduler's FP64 pipe for 64 cycles per warp.  A cluster barrier adds about
+// 1,000 cycles, a hand-over of halo rows about 1,200 (measured: 1,150 on 15
+// CTAs).
+static bool best_shape(int kind, int precision, bool ll, int64_t M, int64_t P, int nt, int G, int maxmem, int B,
+                       double overlap, int max_cluster, TilePlan* out) {
+  if (ll && maxmem > 2) return false;  // members beyond the second: stencil.cu's list
+  const size_t elt = precision == MJP_FP64 ? 8 : 4;
+  const bool row = kind == MJP_BD1D || kind == MJP_TWOSTATE;
+  const int64_t total = kind == MJP_BD1D ? (M + 1) / 2 : kind == MJP_TWOSTATE ? M : kind == MJP_AUTOREG ? P / 2 : (P + 1) / 2;
+  if (!row && M > 768) return false;
+  double best = 0.0;
+  bool found = false;
+  static const int kClusters[] = {1, 2, 3, 4, 6, 8, 10, 12, 14, 16};
+  for (int c : kClusters) {
+    if (c > max_cluster) break;
+    for (const int* rp = runs_of(kind, precision, ll, c > 1); *rp; ++rp) {
+      const int R = *rp, maxt = tile_max_threads(elt, ll, c > 1, R);
+      const int64_t part = (total + c - 1) / c;  // columns or pair rows of a CTA
+      // Grid kinds in a cluster compute halo pair rows of both neighbours and
+      // hand over every `period` jumps.
+      for (int h = 1; h <= (row || c == 1 ? 1 : 3); ++h) {
+        const int halo = row || c == 1 ? 0 : kind == MJP_AUTOREG ? 2 * h : h;
+        const int64_t runs = (part + 2 * halo + R - 1) / R;
+        const int64_t owners = row ? runs : runs * M;
+        if (owners > maxt) continue;
+        const int64_t mine = runs * R - 2 * halo;   // columns or pair rows that are the CTA's own
+        const int C = (int)((total + mine - 1) / mine);  // CTAs that hold something
+        if (C > c || (C == 1) != (c == 1) || mine < halo) continue;
+        TilePlan tp;
+        tp.cluster = C;
+        tp.r = R;
+        tp.geo.tx = (int)(row ? runs : M);
+        tp.geo.ty = (int)(row ? 1 : runs);
+        int64_t threads = (owners + 31) / 32 * 32;
+        tp.gpt = 0;
+        if (ll) {
+          threads = std::max<int64_t>(threads, ((int64_t)G + 8 * 32 - 1) / (8 * 32) * 32);
+          if (threads > maxt) continue;
+          tp.gpt = G <= 2 * threads ? 2 : 8;
+        }
+        tp.threads = (int)threads;
+        const int cells = tile_cells(kind, (int)M, R, tp.geo.tx, tp.geo.ty);
+        if (2 * cells + 1 > 65535) continue;  // tile positions are kept in 16 bits
+        const int J = tile_jumps(elt, R), pairs = R * tp.geo.tx * tp.geo.ty;
+        const int kcmin = ll ? 8 : std::max(8, 2 * J);
+        int kc = 32;
+        while (kc > kcmin && elt * (size_t)nt * (2 * kc + 4) > 40 * 1024) kc /= 2;
+        tp.geo.kc = kc;
+        tp.geo.lgkc = kc == 32 ? 5 : kc == 16 ? 4 : 3;
+        tp.geo.nslot = 0;
+        tp.geo.halo = halo;
+        tp.geo.period = halo == 0 ? 1 << 30 : kind == MJP_AUTOREG ? halo : 2 * halo;
+        const int rows = row ? 0 : tp.geo.ty * R;
+        size_t smem = tile_smem(elt, ll ? 2 : J, cells, nt, kc, ll ? G : 0, 0, pairs, rows, halo * (int)M).total;
+        if (smem > kTileSmemMax) continue;
+        if (!ll) {
+          tp.geo.nslot = smem >= kTileSmemAcc ? 0 : (int)std::min<size_t>((size_t)std::min(nt, 64), (kTileSmemAcc - smem) / ((size_t)pairs * 16));
+          smem = tile_smem(elt, ll ? 2 : J, cells, nt, kc, 0, tp.geo.nslot, pairs, rows, halo * (int)M).total;
+        }
+        tp.smem = smem;
+
+        const double warps = threads / 32.0, gact = ll ? std::ceil((double)G / nt * overlap / threads) : 0.0;
+        double work, lat;
+        if (precision == MJP_FP64) {
+          const double ops = kind == MJP_BD1D ? 6 : kind == MJP_TWOSTATE ? 7 : kind == MJP_MRNA_PROT2D ? 10 : 13;
+          const double per_warp = R * (ops + (ll ? 0.0 : 2.0 * overlap)) + 2.0 * gact;
+          work = warps * per_warp * 16.0;
+          lat = 200.0 + 64.0 * per_warp * (double)((threads / 32 + 3) / 4) + 300.0 * (R - 1);
+        } else {
+          work = warps * (R * (15.0 + (ll ? 0.0 : 4.0 * overlap)) + 5.0 * gact);
+          lat = (row ? 250.0 : 450.0) + work + 15.0 * R;
+        }
+        if (C > 1) lat += halo ? 1200.0 / tp.geo.period : 1000.0;
+        // CTAs of one SM share its pipes; clusters beyond the SMs run in waves.
+        const double per_sm = std::min({65536.0 / (threads * (elt == 4 && R <= 2 ? 80.0 : 128.0)), 227.0 * 1024 / (smem + 1024), 32.0});
+        const double slots = kSms * std::max(1.0, (double)(int)per_sm);
+        const double ctas = (double)B * C;
+        const double waves = std::max(1.0, (double)(int64_t)((ctas + slots - 1) / slots));
+        const double res = std::min(std::max(1.0, ctas / kSms), std::max(1.0, (double)(int)per_sm));
+        const double t = waves * std::max(lat, (precision == MJP_FP64 ? 1.0 : 0.75) * work * res);
+        if (!found || t < best) {
+          best = t;
+          found = true;
+          *out = tp;
+        }
+      }
+    }
+  }
+  return found;
+}
+
+bool tile_plan(int kind, int precision, bool ll, int64_t M, int64_t P, int nt, int G, int maxmem, int B,
+               double overlap, TilePlan* out) {
+  if (!best_shape(kind, precision, ll, M, P, nt, G, maxmem, B, overlap, 16, out)) return false;
+  if (out->cluster <= 8) return true;
+  // More than 8 CTAs only where a GPC holds them.
+  const cudaError_t e = precision == MJP_FP64 ? (ll ? tile_ll64(kind, nullptr, *out, 0) : tile_ex64(kind, nullptr, *out, 0))
+                                              : (ll ? tile_ll32(kind, nullptr, *out, 0) : tile_ex32(kind, nullptr, *out, 0));
+  if (e == cudaSuccess) return true;
+  cudaGetLastError();
+  return best_shape(kind, precision, ll, M, P, nt, G, maxmem, B, overlap, 8, out);
+}
+
+cudaError_t launch_chain_tile(int kind, int precision, bool ll, const ChainParams& p, const TilePlan& tp,
+                              cudaStream_t s) {
+  if (precision == MJP_FP64) return ll ? tile_ll64(kind, &p, tp, s) : tile_ex64(kind, &p, tp, s);
+  return ll ? tile_ll32(kind, &p, tp, s) : tile_ex32(kind, &p, tp, s);
+}
+
+}  // namespace mjp
