@@ -110,7 +110,8 @@ extern "C" {
                                    of FP32 two-state models whose observation groups have at most two members (one
                                    CTA of MJP_OPT_THREADS / 32 <= 8 warps per theta; automatic when 0) and for
                                    expv_series of birth-death models (automatic thread count), none with a forced
-                                   cluster size; else, without a forced thread count or cluster size, the kernel with
+                                   cluster size; expv_series of birth-death and two-state models of at most 512
+                                   states: one state per thread; else, without a forced thread count or cluster size, the kernel with
                                    registers and a shared-memory tile (groups of at most two members), else the
                                    shared-memory kernel), 1 = shared-memory
                                    kernel, 2 = register-resident kernel (MJP_ERR_UNSUPPORTED where it does not

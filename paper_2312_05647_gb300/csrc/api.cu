@@ -742,12 +742,17 @@ int expv_series(mjp_model* m, const void* rho0, const double* times, int ntimes,
     return MJP_OK;
   }
 
-  // Birth-death chains: the register-resident kernel (one CTA, or the fewest
-  // CTAs of a cluster that hold the chain, halo 32) unless a thread count is
-  // asked for.
+  // Small birth-death and two-state models at the automatic shape: one state
+  // per thread.  Other birth-death chains: the register-resident kernel (one
+  // CTA, or the fewest CTAs of a cluster that hold the chain, halo 32) unless a
+  // thread count is asked for.
   Reg1dPlan rp1 = {};
   bool use_reg1 = false;
-  if (m->kind == MJP_BD1D && m->chain != 1 && m->threads == 0) {
+  SmallPlan sp = {};
+  const bool automatic = m->chain == 0 && m->cluster == 0 && m->threads == 0 && m->kcap <= (1 << 30) - 1;
+  const double overlap = automatic ? window_overlap(m, st.data(), nt) : 0.0;
+  const bool use_small = automatic && chain_small_plan(m->kind, m->precision, m->M, m->N, nt, overlap, &sp);
+  if (!use_small && m->kind == MJP_BD1D && m->chain != 1 && m->threads == 0) {
     const int c0 = m->cluster > 0 ? m->cluster : 1, c1 = m->cluster > 0 ? m->cluster : 8;
     for (int c = c0; c <= c1 && !use_reg1; ++c) use_reg1 = chain_reg1d_plan(m->precision, m->N, nt, c, 32, &rp1, true);
   }
@@ -756,19 +761,19 @@ int expv_series(mjp_model* m, const void* rho0, const double* times, int ntimes,
                                      "a forced thread count that fits 8 CTAs");
   // Other models at the automatic shape: the register/tile chain, where it fits.
   TilePlan xp = {};
-  const bool use_tile = !use_reg1 && m->chain == 0 && m->cluster == 0 && m->threads == 0 && m->kcap <= (1 << 30) - 1 &&
-                        tile_plan(m->kind, m->precision, false, m->M, m->P, nt, 0, 0, 1, window_overlap(m, st.data(), nt), &xp);
+  const bool use_tile = !use_small && !use_reg1 && automatic &&
+                        tile_plan(m->kind, m->precision, false, m->M, m->P, nt, 0, 0, 1, overlap, &xp);
   int C = 0, T = 0;
   int64_t slab = 0;
   int rc = 0;
-  if (!use_reg1 && !use_tile && (rc = stencil_config(m, 0, nt, 0, 0, &C, &T, &slab))) return rc;
+  if (!use_small && !use_reg1 && !use_tile && (rc = stencil_config(m, 0, nt, 0, 0, &C, &T, &slab))) return rc;
   if ((rc = ensure_status(m))) return rc;
   if ((rc = m->d_times.ensure(sizeof(double) * nt))) return rc;
   if ((rc = m->d_orig.ensure(sizeof(int32_t) * nt))) return rc;
   if ((rc = m->d_win.ensure(sizeof(Win) * nt))) return rc;
   if ((rc = m->d_info.ensure(sizeof(JobInfo)))) return rc;
   if ((rc = m->d_theta.ensure(sizeof(double) * m->theta.size()))) return rc;
-  if (!use_reg1 && m->precision == MJP_FP32 && (rc = m->d_comp.ensure(sizeof(float) * (size_t)nt * m->N))) return rc;
+  if (!use_small && !use_reg1 && m->precision == MJP_FP32 && (rc = m->d_comp.ensure(sizeof(float) * (size_t)nt * m->N))) return rc;
   MJP_CUDA(cudaMemcpyAsync(m->d_times.p, st.data(), sizeof(double) * nt, cudaMemcpyHostToDevice, s));
   MJP_CUDA(cudaMemcpyAsync(m->d_orig.p, order.data(), sizeof(int32_t) * nt, cudaMemcpyHostToDevice, s));
   MJP_CUDA(cudaMemcpyAsync(m->d_theta.p, m->theta.data(), sizeof(double) * m->theta.size(), cudaMemcpyHostToDevice, s));
@@ -793,7 +798,8 @@ int expv_series(mjp_model* m, const void* rho0, const double* times, int ntimes,
   cp.out = out; cp.out_stride = 0; cp.comp = m->d_comp.as<float>(); cp.comp_stride = 0;
   cp.renorm = (m->precision == MJP_FP32) ? m->renorm : 0;
   cp.slab = slab; cp.status = pp.status; cp.wait_limit = m->wait_limit;
-  if (use_reg1) MJP_CUDA(launch_chain_reg1d(m->precision, cp, rp1, s));
+  if (use_small) MJP_CUDA(launch_chain_small(m->kind, m->precision, cp, sp, s));
+  else if (use_reg1) MJP_CUDA(launch_chain_reg1d(m->precision, cp, rp1, s));
   else if (use_tile) MJP_CUDA(launch_chain_tile(m->kind, m->precision, false, cp, xp, s));
   else MJP_CUDA(launch_chain_stencil(m->kind, m->precision, 0, cp, C, T, s));
   if ((rc = mark(m, 2, s))) return rc;

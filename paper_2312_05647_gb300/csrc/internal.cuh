@@ -222,6 +222,16 @@ struct RegTsPlan {
 bool chain_regts_plan(int64_t M, int ntimes, int G, int maxmem, int col_lo, int col_hi, int threads,
                       RegTsPlan* out);
 cudaError_t launch_chain_regts(const ChainParams& p, const RegTsPlan& rp, cudaStream_t s);
+// Transient distributions of small birth-death and two-state models
+// (stencil_small.cu): one CTA, one state per thread, reducer warps.
+struct SmallPlan {
+  int nchain;    // threads of the chain (whole warps)
+  int threads;   // with the reducers
+  size_t smem;
+};
+// overlap: windows that hold a jump, on average.
+bool chain_small_plan(int kind, int precision, int64_t M, int64_t N, int nt, double overlap, SmallPlan* out);
+cudaError_t launch_chain_small(int kind, int precision, const ChainParams& p, const SmallPlan& sp, cudaStream_t s);
 int64_t rk4_max_states();
 // Krylov subspace steps for one birth-death distribution (krylov.cu).
 struct KrylovParams {
