@@ -241,28 +241,42 @@ int arena_prepare(mjp_model* m, const double* host_theta, int B, const double* t
   return MJP_OK;
 }
 
-// The general-CSR chain: planner, windows back to the host (the number of
-// launches is the largest K), weight table, rho0 into the in-degree order,
-// then one launch per jump.  Leaves the outputs (times in ascending order,
-// states in the internal order) in m->d_outp.
+// The general-CSR chain: planner (which also forms the weight table), windows
+// back to the host (the number of launches is the largest K), rho0 into the
+// in-degree order, then one launch per jump and one per kCsrBlock jumps for the
+// outputs.  Leaves the outputs (times in ascending order, states in the
+// internal order) in m->d_outp.
 int csr_run(mjp_model* m, const void* rho0, const double* sorted_times, int nt, int trunc_mode, double tol,
             cudaStream_t s, std::vector<Win>* wins) {
   const size_t elt = m->precision == MJP_FP64 ? 8 : 4;
   const int64_t n = m->N;
+  // The ring of vectors: a block of jumps and the one being formed; two
+  // vectors where nine would take more than 16 GiB (and for the one-launch chain).
+  const int block = m->chain == 2 || (size_t)(kCsrBlock + 1) * elt * n > ((size_t)16 << 30) ? 1 : kCsrBlock;
+  const int nring = block + 1;
+  // Weights of a window: at most 20 sqrt(x) + 16 (x - 10 sqrt x .. x + 10 sqrt x + 10).
+  double wcap = 2.0;
+  // (Windows beyond the cap are refused below.)
+  for (int i = 0; i < nt; ++i) wcap += 20.0 * std::sqrt(std::min(m->csr_omega * sorted_times[i], (double)m->kcap)) + 16.0;
+  const int64_t wtab = (int64_t)wcap;
   int rc = 0;
   if ((rc = ensure_status(m)) || (rc = m->d_times.ensure(sizeof(double) * nt)) ||
       (rc = m->d_win.ensure(sizeof(Win) * nt)) || (rc = m->d_info.ensure(sizeof(JobInfo))) ||
-      (rc = m->d_rho2.ensure(2 * elt * n)) || (rc = m->d_outp.ensure(elt * (size_t)nt * n)) ||
+      (rc = m->d_rho2.ensure((size_t)nring * elt * n)) || (rc = m->d_outp.ensure(elt * (size_t)nt * n)) ||
       (rc = m->d_woff.ensure(sizeof(int64_t) * nt)) || (rc = m->d_L.ensure(sizeof(int64_t) * nt)) ||
-      (rc = m->d_K.ensure(sizeof(int64_t) * nt)))
+      (rc = m->d_K.ensure(sizeof(int64_t) * nt)) || (rc = m->d_wtab.ensure(sizeof(double) * (size_t)(wtab + 2))) ||
+      (rc = m->d_arena_ctl.ensure(16)))
     return rc;
   if (m->precision == MJP_FP32 && (rc = m->d_comp.ensure(sizeof(float) * (size_t)nt * n))) return rc;
   MJP_CUDA(cudaMemcpyAsync(m->d_times.p, sorted_times, sizeof(double) * nt, cudaMemcpyHostToDevice, s));
+  MJP_CUDA(cudaMemsetAsync(m->d_arena_ctl.p, 0, 16, s));
   PlanParams pp = {};
   pp.kind = MJP_CSR; pp.M = 1; pp.P = 1; pp.N = n; pp.ntheta = 0; pp.theta = nullptr; pp.B = 1;
   pp.ntimes = nt; pp.times = m->d_times.as<double>();
   pp.trunc_mode = trunc_mode; pp.tol = tol; pp.omega_factor = 1.1; pp.omega_fixed = m->csr_omega;
-  pp.fp64_weights = m->precision == MJP_FP64 ? 1 : 0;
+  pp.fp64_weights = 1; pp.arena_fp64 = 1;
+  pp.arena = m->d_wtab.p; pp.arena_cap = wtab;
+  pp.arena_used = m->d_arena_ctl.as<unsigned long long>();
   pp.kcap = m->kcap; pp.win = m->d_win.as<Win>(); pp.info = m->d_info.as<JobInfo>();
   pp.status = m->d_status.as<int>();
   if ((rc = mark(m, 0, s))) return rc;
@@ -276,40 +290,42 @@ int csr_run(mjp_model* m, const void* rho0, const double* sorted_times, int nt, 
     MJP_CUDA(cudaMemset(m->d_status.p, 0, sizeof(int)));
     return map_status(st);
   }
+  // Windows without a stored copy: t = 0 or no transitions (P_0 = 1, P_1 = 0).
+  const double start[2] = {1.0, 0.0};
+  MJP_CUDA(cudaMemcpyAsync(m->d_wtab.as<double>() + wtab, start, sizeof(start), cudaMemcpyHostToDevice, s));
   std::vector<int64_t> woff(nt), L(nt), K(nt);
-  int64_t tot = 0, kmax = 0;
+  int64_t kmax = 0;
   for (int i = 0; i < nt; ++i) {
-    woff[i] = tot;
-    L[i] = (*wins)[i].L;
-    K[i] = (*wins)[i].K;
-    tot += K[i] - L[i] + 1;
+    const Win& w = (*wins)[i];
+    if (w.woff < 0 && w.x != 0.0) return fail(MJP_ERR_CUDA, "weight table too small");
+    woff[i] = w.woff >= 0 ? w.woff : wtab;
+    L[i] = w.L;
+    K[i] = w.K;
     kmax = std::max(kmax, K[i]);
   }
-  if ((rc = m->d_wtab.ensure(sizeof(double) * std::max<int64_t>(tot, 1)))) return rc;
   MJP_CUDA(cudaMemcpyAsync(m->d_woff.p, woff.data(), sizeof(int64_t) * nt, cudaMemcpyHostToDevice, s));
   MJP_CUDA(cudaMemcpyAsync(m->d_L.p, L.data(), sizeof(int64_t) * nt, cudaMemcpyHostToDevice, s));
   MJP_CUDA(cudaMemcpyAsync(m->d_K.p, K.data(), sizeof(int64_t) * nt, cudaMemcpyHostToDevice, s));
-  MJP_CUDA(launch_fill_weights(m->d_win.as<Win>(), nt, m->d_woff.as<int64_t>(), m->d_wtab.as<double>(), s));
   char* rho = m->d_rho2.as<char>();
   MJP_CUDA(launch_permute_in(m->precision, rho0, m->d_perm.as<int32_t>(), rho, n, s));
   if ((rc = mark(m, 1, s))) return rc;
-  CsrJumpParams jp = {};
-  jp.n = n; jp.nslices = m->nslices;
-  jp.slice_ptr = m->d_slice_ptr.as<int64_t>(); jp.slice_len = m->d_slice_len.as<int32_t>();
-  jp.col = m->d_col.as<int32_t>(); jp.val = m->d_val.p; jp.diag = m->d_diag.p;
-  jp.wtab = m->d_wtab.as<double>(); jp.woff = m->d_woff.as<int64_t>();
-  jp.L = m->d_L.as<int64_t>(); jp.K = m->d_K.as<int64_t>();
-  jp.out = m->d_outp.p; jp.comp = m->d_comp.as<float>();
   if (m->chain == 2) {
     // The whole chain in one cooperative launch, jumps separated by a
     // bounded grid barrier (a wait that runs out is reported by
     // rate_model_check as MJP_ERR_DEVICE_TIMEOUT).  Measured slower than
     // one launch per jump at N = 2^20 (12.6 against 11.4 ms for 309 jumps,
-    // FP32): the barrier costs more than the gap between launches.
+    // FP32, before those launches overlapped): the barrier costs more than the
+    // gap between launches.
     if ((rc = m->d_bar.ensure(2 * sizeof(unsigned)))) return rc;
     MJP_CUDA(cudaMemsetAsync(m->d_bar.p, 0, 2 * sizeof(unsigned), s));
     CsrChainParams cp = {};
-    cp.j = jp;
+    CsrJumpParams& jp = cp.j;
+    jp.n = n; jp.nslices = m->nslices;
+    jp.slice_ptr = m->d_slice_ptr.as<int64_t>(); jp.slice_len = m->d_slice_len.as<int32_t>();
+    jp.col = m->d_col.as<int32_t>(); jp.val = m->d_val.p; jp.diag = m->d_diag.p;
+    jp.wtab = m->d_wtab.as<double>(); jp.woff = m->d_woff.as<int64_t>();
+    jp.L = m->d_L.as<int64_t>(); jp.K = m->d_K.as<int64_t>();
+    jp.out = m->d_outp.p; jp.comp = m->d_comp.as<float>();
     cp.ntimes = nt;
     cp.kmax = kmax;
     cp.rho = rho;
@@ -318,18 +334,31 @@ int csr_run(mjp_model* m, const void* rho0, const double* sorted_times, int nt, 
     cp.status = m->d_status.as<int>();
     MJP_CUDA(launch_csr_chain(m->precision, cp, s));
   } else {
-    int lo = 0, hi = -1;  // times whose window holds jump k-1 (ascending times)
-    for (int64_t k = 1; k <= kmax + 1; ++k) {
-      const int64_t kp = k - 1;
-      while (lo < nt && K[lo] < kp) ++lo;
-      while (hi + 1 < nt && L[hi + 1] <= kp) ++hi;
-      jp.k = k;
-      jp.jump = k <= kmax;
-      jp.tlo = lo;
-      jp.thi = hi;
-      jp.rho_prev = rho + ((kp & 1) ? elt * n : 0);
-      jp.rho_next = rho + ((kp & 1) ? 0 : elt * n);
-      MJP_CUDA(launch_csr_jump(m->precision, jp, s));
+    CsrStepParams jp = {};
+    jp.n = n;
+    jp.slice_ptr = m->d_slice_ptr.as<int64_t>(); jp.slice_len = m->d_slice_len.as<int32_t>();
+    jp.col = m->d_col.as<int32_t>(); jp.val = m->d_val.p; jp.diag = m->d_diag.p;
+    CsrSumParams sp = {};
+    sp.n = n; sp.nring = nring; sp.ring = rho;
+    sp.wtab = m->d_wtab.as<double>(); sp.woff = m->d_woff.as<int64_t>();
+    sp.L = m->d_L.as<int64_t>(); sp.K = m->d_K.as<int64_t>();
+    sp.out = m->d_outp.p; sp.comp = m->d_comp.as<float>();
+    int lo = 0, hi = -1;  // times whose window meets the block (ascending times)
+    for (int64_t k = 0; k <= kmax; ++k) {
+      if (k > 0) {
+        jp.rho_prev = rho + (size_t)((k - 1) % nring) * elt * n;
+        jp.rho_next = rho + (size_t)(k % nring) * elt * n;
+        MJP_CUDA(launch_csr_step(m->precision, jp, s));
+      }
+      if ((k + 1) % block != 0 && k != kmax) continue;
+      sp.k0 = k / block * block;
+      sp.count = (int)(k - sp.k0 + 1);
+      while (lo < nt && K[lo] < sp.k0) ++lo;
+      while (hi + 1 < nt && L[hi + 1] <= k) ++hi;
+      if (lo > hi) continue;
+      sp.tlo = lo;
+      sp.thi = hi;
+      MJP_CUDA(launch_csr_sum(m->precision, sp, s));
     }
   }
   if ((rc = mark(m, 2, s))) return rc;

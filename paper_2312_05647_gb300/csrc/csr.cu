@@ -12,17 +12,26 @@
 // separate array.  rho (4 MB for 2^20 FP32 states) stays resident in L2;
 // neighbour values are gathered with read-only loads.
 //
-// Jump k accumulates rho_{k-1} into the active times' outputs
-// (Kahan-compensated in FP32) and forms rho_k = rho_{k-1} B (Algorithm 2's
-// loop body); rho_{k+1} depends on all of rho_k, so jumps are separated grid-
-// wide.  Default: one launch per jump.  Alternative (MJP_OPT_CHAIN = 2): the
-// whole chain in one cooperative launch (all CTAs co-resident), jumps
+// Default: one launch per jump (rho_k = rho_{k-1} B, Algorithm 2's loop body;
+// rho_{k+1} depends on all of rho_k, so jumps are separated grid-wide).  Each
+// launch may begin while the one before it ends (programmatic dependent
+// launch): indices, rates and the diagonal, which do not depend on it, are
+// loaded first, so that only the gathers and the multiply-adds follow the wait.
+// The last 8 (kCsrBlock) jumps stay in a ring of vectors, and one launch per 8
+// jumps adds their terms P_k rho_k to the active times' outputs (FP32: a Kahan
+// step per jump), instead of every jump reading and writing every active
+// output.
+//
+// Alternative (MJP_OPT_CHAIN = 2): the whole chain in one cooperative launch
+// (all CTAs co-resident), the outputs accumulated at every jump, jumps
 // separated by a software grid barrier whose waits are bounded (a CTA that
 // polls longer than the limit records kStatusTimeout and leaves, and so do
-// the others at their next barrier).  Both run the same per-jump code, so
-// their results are identical.  The Poisson weights of every (time, jump)
-// come from a table filled by `fill_weights_kernel` with Algorithm 2's
-// recurrence P_k = P_{k-1} x/k started from the planner's P_L.
+// the others at their next barrier).  The arithmetic is the same.  The
+// Poisson weights of every (time, jump) are the planner's, in FP64.
+//
+// Bound: one 4-byte gather per lane costs the L1 a tag look-up of its own, one
+// a cycle and SM (measured peak 320 G/s), for large matrices; for small ones
+// the latency of a launch and of a gather.
 #include <algorithm>
 
 #include "internal.cuh"
@@ -35,20 +44,6 @@ __device__ __forceinline__ float fma_t(float a, float b, float c) { return __fma
 __device__ __forceinline__ double fma_t(double a, double b, double c) { return __fma_rn(a, b, c); }
 __device__ __forceinline__ float mul_t(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double mul_t(double a, double b) { return __dmul_rn(a, b); }
-
-// One warp per time: table[i][k - L_i] = P_k for k in [L_i, K_i], with the
-// tail 1 - sum P folded into the last entry.
-__global__ void fill_weights_kernel(const Win* win, int ntimes, const int64_t* woff, double* table) {
-  int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (i >= ntimes || (threadIdx.x & 31) != 0) return;
-  Win w = win[i];
-  double* t = table + woff[i];
-  double P = w.PL;
-  for (int64_t k = w.L; k <= w.K; ++k) {
-    if (k > w.L) P = __dmul_rn(P, __ddiv_rn(w.x, (double)k));
-    t[k - w.L] = (k == w.K) ? P + w.tail : P;
-  }
-}
 
 template <typename T>
 __global__ void permute_in_kernel(const T* __restrict__ src, const int32_t* __restrict__ perm, T* __restrict__ dst,
@@ -141,9 +136,99 @@ __device__ __forceinline__ void csr_jump_body(const CsrJumpParams& p) {
   }
 }
 
+// One jump, a thread per state: its first kCsrPre entries are in registers
+// before the wait, and the next ones are loaded while the last ones' gathers
+// are on their way.  The multiply-adds run in entry order, as in csr_jump_body.
+constexpr int kCsrPre = 8;
 template <typename T>
-__global__ void __launch_bounds__(512) csr_jump_kernel(CsrJumpParams p) {
-  csr_jump_body<T>(p);
+__global__ void __launch_bounds__(256) csr_step_kernel(const CsrStepParams p) {
+  const int64_t r = blockIdx.x * (int64_t)256 + threadIdx.x;
+  const bool valid = r < p.n;
+  const int64_t s = valid ? r >> 5 : 0;
+  const int64_t base = p.slice_ptr[s] + (threadIdx.x & 31);
+  const int width = valid ? p.slice_len[s] : 0;
+  const int32_t* col = p.col + base;
+  const T* val = reinterpret_cast<const T*>(p.val) + base;
+  const T dg = valid ? reinterpret_cast<const T*>(p.diag)[r] : (T)0;
+  const T* rho = reinterpret_cast<const T*>(p.rho_prev);  // (written by the launch before: no read-only loads)
+  int32_t c[kCsrPre];
+  T a[kCsrPre];
+  auto fetch = [&](int j0) {
+#pragma unroll
+    for (int u = 0; u < kCsrPre; ++u)
+      if (j0 + u < width) {
+        c[u] = __ldcs(col + (int64_t)(j0 + u) * 32);
+        a[u] = __ldcs(val + (int64_t)(j0 + u) * 32);
+      }
+  };
+  fetch(0);
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
+  if (!valid) return;
+  T y = mul_t(dg, rho[r]);
+  for (int j0 = 0; j0 < width; j0 += kCsrPre) {
+    T g[kCsrPre], w[kCsrPre];
+#pragma unroll
+    for (int u = 0; u < kCsrPre; ++u)
+      if (j0 + u < width) {
+        g[u] = rho[c[u]];
+        w[u] = a[u];
+      }
+    if (j0 + kCsrPre < width) fetch(j0 + kCsrPre);
+#pragma unroll
+    for (int u = 0; u < kCsrPre; ++u)
+      if (j0 + u < width) y = fma_t(w[u], g[u], y);
+  }
+  reinterpret_cast<T*>(p.rho_next)[r] = y;
+}
+
+// out_i += P_k rho_k for k = k0 .. k0 + count - 1 (count <= kCsrBlock) inside
+// the window of time i, for the times [tlo, thi], whose windows meet the block.
+template <typename T>
+__global__ void __launch_bounds__(256) csr_sum_kernel(const CsrSumParams p) {
+  __shared__ double ws[kCsrBlock];
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
+  const int64_t r = blockIdx.x * (int64_t)256 + threadIdx.x;
+  const bool valid = r < p.n;
+  const T* ring = reinterpret_cast<const T*>(p.ring);
+  T h[kCsrBlock];
+#pragma unroll
+  for (int j = 0; j < kCsrBlock; ++j)
+    h[j] = valid && j < p.count ? ring[(size_t)((p.k0 + j) % p.nring) * p.n + r] : (T)0;
+  for (int i = p.tlo; i <= p.thi; ++i) {
+    const int64_t L = p.L[i], K = p.K[i];
+    __syncthreads();
+    if (threadIdx.x < kCsrBlock) {
+      const int64_t k = p.k0 + threadIdx.x;
+      ws[threadIdx.x] = (int)threadIdx.x < p.count && k >= L && k <= K ? p.wtab[p.woff[i] + (k - L)] : 0.0;
+    }
+    __syncthreads();
+    if (!valid) continue;
+    T* o = reinterpret_cast<T*>(p.out) + (size_t)i * p.n + r;
+    const bool first = L >= p.k0, last = K < p.k0 + p.count;
+    // The steps of csr_jump_body, a block of them on registers.
+    const int j0 = first ? (int)(L - p.k0) : 0, j1 = last ? (int)(K - p.k0) : p.count - 1;
+    T sum = first ? (T)0 : *o;
+    if constexpr (sizeof(T) == 4) {
+      float* cp = p.comp + (size_t)i * p.n + r;
+      float c = first ? 0.0f : *cp;
+#pragma unroll
+      for (int j = 0; j < kCsrBlock; ++j) {
+        if (j < j0 || j > j1) continue;
+        const float y = __fsub_rn(__fmul_rn((float)ws[j], h[j]), c), t = __fadd_rn(sum, y);
+        c = __fsub_rn(__fsub_rn(t, sum), y);
+        sum = t;
+      }
+      *o = last ? __fsub_rn(sum, c) : sum;
+      if (!last) *cp = c;
+    } else {
+#pragma unroll
+      for (int j = 0; j < kCsrBlock; ++j)
+        if (j >= j0 && j <= j1) sum = fma_t(ws[j], h[j], sum);
+      *o = sum;
+    }
+  }
 }
 
 // Grid-wide barrier with a bounded wait.  bar[0] counts arrivals, bar[1] is
@@ -245,11 +330,6 @@ int grid_for(int64_t work, int block) {
 
 }  // namespace
 
-cudaError_t launch_fill_weights(const Win* win, int ntimes, const int64_t* woff, double* table, cudaStream_t s) {
-  fill_weights_kernel<<<(ntimes + 7) / 8, 256, 0, s>>>(win, ntimes, woff, table);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_permute_in(int precision, const void* src, const int32_t* perm, void* dst, int64_t n,
                               cudaStream_t s) {
   if (precision == MJP_FP64)
@@ -270,12 +350,31 @@ cudaError_t launch_permute_out(int precision, const void* src, const int32_t* pe
   return cudaGetLastError();
 }
 
-cudaError_t launch_csr_jump(int precision, const CsrJumpParams& p, cudaStream_t s) {
-  const int block = 512;
-  int grid = grid_for(p.nslices * 32, block);
-  if (precision == MJP_FP64) csr_jump_kernel<double><<<grid, block, 0, s>>>(p);
-  else csr_jump_kernel<float><<<grid, block, 0, s>>>(p);
-  return cudaGetLastError();
+// Launch that may begin while the one before it in the stream ends.
+template <typename P>
+static cudaError_t launch_dependent(void (*kern)(P), int64_t grid, const P& p, cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(256);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, p);
+}
+
+cudaError_t launch_csr_step(int precision, const CsrStepParams& p, cudaStream_t s) {
+  const int64_t grid = (p.n + 255) / 256;
+  return precision == MJP_FP64 ? launch_dependent(csr_step_kernel<double>, grid, p, s)
+                               : launch_dependent(csr_step_kernel<float>, grid, p, s);
+}
+
+cudaError_t launch_csr_sum(int precision, const CsrSumParams& p, cudaStream_t s) {
+  const int64_t grid = (p.n + 255) / 256;
+  return precision == MJP_FP64 ? launch_dependent(csr_sum_kernel<double>, grid, p, s)
+                               : launch_dependent(csr_sum_kernel<float>, grid, p, s);
 }
 
 template <typename T>

@@ -120,7 +120,36 @@ struct ChainParams {
   long long wait_limit = 1LL << 24;
 };
 
-// One jump of the general-CSR chain (csr.cu).
+constexpr int kCsrBlock = 8;  // jumps the general-CSR chain keeps before it adds them to the outputs
+
+// One launch of the general-CSR chain (csr.cu): rho_next = rho_prev B.
+struct CsrStepParams {
+  int64_t n;
+  const int64_t* slice_ptr;  // first entry of each slice
+  const int32_t* slice_len;  // entries per state in each slice
+  const int32_t* col;        // permuted source state of each entry
+  const void* val;           // lambda / Omega (T)
+  const void* diag;          // 1 - e_n / Omega (T)
+  const void* rho_prev;
+  void* rho_next;
+};
+// The sums of a block of jumps k0 .. k0 + count - 1 (count <= kCsrBlock); rho_k
+// lies in vector k mod nring of the ring.
+struct CsrSumParams {
+  int64_t n;
+  int64_t k0;
+  int count, nring;
+  const void* ring;
+  int tlo, thi;              // times whose window meets the block
+  const double* wtab;        // weights table
+  const int64_t* woff;       // table offset per time
+  const int64_t* L;          // window start per time
+  const int64_t* K;          // window end per time
+  void* out;                 // ntimes x n outputs (T, permuted order)
+  float* comp;               // FP32 Kahan compensation, ntimes x n
+};
+
+// One jump of the general-CSR chain in one launch (csr.cu).
 struct CsrJumpParams {
   int64_t n, nslices;
   const int64_t* slice_ptr;  // first entry of each slice
@@ -274,12 +303,12 @@ int krylov_max_states();
 int krylov_max_kappa();
 cudaError_t launch_krylov(const KrylovParams& p, cudaStream_t s);
 cudaError_t launch_rk4(const Rk4Params& p, cudaStream_t s);
-cudaError_t launch_fill_weights(const Win* win, int ntimes, const int64_t* woff, double* table, cudaStream_t s);
 cudaError_t launch_permute_in(int precision, const void* src, const int32_t* perm, void* dst, int64_t n,
                               cudaStream_t s);
 cudaError_t launch_permute_out(int precision, const void* src, const int32_t* perm, void* dst, int64_t n,
                                int ntimes, const int32_t* orig, cudaStream_t s);
-cudaError_t launch_csr_jump(int precision, const CsrJumpParams& p, cudaStream_t s);
+cudaError_t launch_csr_step(int precision, const CsrStepParams& p, cudaStream_t s);
+cudaError_t launch_csr_sum(int precision, const CsrSumParams& p, cudaStream_t s);
 cudaError_t launch_csr_chain(int precision, const CsrChainParams& p, cudaStream_t s);
 cudaError_t launch_csr_loglik(const void* outp, int precision, int64_t n, const int64_t* gptr, int ntimes,
                               const double* counts, const int64_t* mptr, const int32_t* members,
