@@ -1,15 +1,32 @@
 // plan.cu -- the FP64 planner: Omega, truncation index K and Poisson weight
 // window of every (instance, time) pair (Eq. B_def, Algorithm 2).
 //
-// One CTA per instance.  Omega = 1.1 max_n e_n is a block max-reduction over
-// the matrix-free exit rates (stencil models) or taken from the model (CSR).
-// Each warp then plans one time: K = floor(x + 6 sqrt x) + 1 with x = Omega t
-// computed with exactly the roundings of Algorithm 2 (no fused multiply-add),
-// and the Poisson weights around the mode m = floor(x) as ratios to w_m = 1,
-// formed by warp-shuffle inclusive product scans of x/k (upwards) and
-// (k+1)/x (downwards).  No exp(-x) is ever formed, so nothing underflows; the
-// window sum W normalises the weights, and the tail mass beyond K is summed
-// explicitly (equal to 1 - sum_{k<=K} P_k, Algorithm 2's last line).
+// One CTA per instance (one per window for a single instance).  Omega = 1.1
+// max_n e_n: the exit rates grow with every coordinate up to the last but one
+// state of an axis (sums of rounded non-negative terms are monotone), so the
+// maximum is among the corners of the box (stencil models), or taken from the
+// model (CSR).
+//
+// Paper's rule, in four phases.  A thread per window: K = floor(x + 6 sqrt x)
+// + 1 with x = Omega t computed with exactly the roundings of Algorithm 2 (no
+// fused multiply-add), the window's bounds and its place in the weight store.
+// A warp per window and direction: the Poisson weights around the mode m =
+// floor(x) as ratios to w_m = 1, x/k upwards and (k+1)/x downwards, as running
+// products of 8 terms per lane joined by a warp-wide product scan.  A thread
+// per window: the sum W that normalises the weights, the tail beyond K summed
+// explicitly (equal to 1 - sum_{k<=K} P_k, Algorithm 2's last line).  A warp
+// per window: the stored weights scaled.  No exp(-x) is ever formed, so nothing
+// underflows.
+//
+// Bound: the FP64 pipe (16 cycles per warp instruction and SM).  Work that all
+// lanes of a warp did alike (roots and divisions, about 250 instructions per
+// window) runs a thread per window instead, and the FP64 reciprocals of 8
+// consecutive k are one reciprocal of their product and 8 multiplications.
+// Measured: 256 thetas x 50 times FP32 151 -> 117 us, 10^4 thetas x 5 times
+// FP64 756 -> 567 us, one theta x 5 times FP64 20 -> 12 us.
+//
+// Tolerance rule: a warp per window does everything (K is known only after the
+// scans).
 #include "internal.cuh"
 
 namespace mjp {
@@ -107,6 +124,20 @@ __device__ bool window_bounds(const PlanParams& p, double x, int64_t& L, int64_t
   return true;
 }
 
+// A window whose K is above the cap: a NaN weight makes this time's result
+// (and a log-likelihood using it) NaN, so a caller that keeps going (a
+// sampler) rejects the parameters.
+__device__ Win capped_window(double x) {
+  Win r;
+  r.x = x;
+  r.L = 0;
+  r.K = 0;
+  r.PL = __longlong_as_double(0x7ff8000000000000LL);
+  r.tail = 0.0;
+  r.woff = -1;
+  return r;
+}
+
 // Float-float numbers (hi + lo, |lo| <= ulp(hi) / 2: ~48 significant bits)
 // on the FP32 pipe, which GB300 runs 64 times faster than its FP64 pipe.
 // Error-free transformations: TwoSum (Knuth), FastTwoSum (Dekker, |a| >= |b|)
@@ -155,16 +186,19 @@ __device__ __forceinline__ FF ff_shfl_up(FF a, int d) {
   return FF{__shfl_up_sync(kFull, a.hi, d), __shfl_up_sync(kFull, a.lo, d)};
 }
 
-// Weights of the paper's rule, ratios to w_m = 1 at the mode m = floor(x):
-// upward w_k = w_{k-1} x / k over (m, R], downward w_k = w_{k+1} (k+1) / x
-// over [L, m).  Each lane forms the running product of a run of kRun
-// consecutive terms, one warp-wide product scan joins the runs.  The
-// products run in float-float (relative error ~1e-14 over a window of ~10^4
-// terms: far below the FP32 weights the chains read and the 1e-12 of the FP64
-// chains are served by paper_weights64), and so do the per-lane sums.  Returns the window sum W over [L, R],
-// the tail sum over (K, R] and w_L; the unnormalised weights of [L, K] go to
-// `put` when `store`.
+// Weights of the paper's rule, ratios to w_m = 1 at the mode m = floor(x), in
+// one direction: upward w_k = w_{k-1} x / k over (m, R] (dir 0), downward
+// w_k = w_{k+1} (k+1) / x over [L, m) (dir 1).  Each lane forms the running
+// product of a run of kRun consecutive terms, one warp-wide product scan joins
+// the runs.  The unnormalised weights of [L, K] go to `put` when `store`;
+// returns (lane 0) the sum of all weights, that of k > K and, downward, w_L.
+//
+// FP32 chains: products and sums in float-float (relative error ~1e-14 over a
+// window of ~10^4 terms, far below the FP32 weights the chains read).
 constexpr int kRun = 8;
+struct FFSums {
+  FF all, tail, wL;
+};
 __device__ __forceinline__ FF ff_warp_incl_prod(FF v, int lane) {
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -173,222 +207,191 @@ __device__ __forceinline__ FF ff_warp_incl_prod(FF v, int lane) {
   }
   return v;
 }
+__device__ __forceinline__ FF ff_warp_sum(FF v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+    v = ff_add(v, FF{__shfl_xor_sync(kFull, v.hi, o), __shfl_xor_sync(kFull, v.lo, o)});
+  return v;
+}
 template <class Put>
-__device__ void paper_weights(double x, int64_t L, int64_t K, int64_t m, int64_t R, int lane, bool store,
-                              Put& put, double& W, double& tailsum, double& wL) {
-  FF sw{lane == 0 ? 1.0f : 0.0f, 0.0f}, st{0.0f, 0.0f}, wl{0.0f, 0.0f};
-  if (store && lane == 0) put(m, FF{1.0f, 0.0f});
-  const FF xf = ff_from(x), invx = ff_from(1.0 / x);
+__device__ FFSums dir_weights(int dir, double x, double invxd, int64_t L, int64_t K, int64_t m, int64_t R, int lane,
+                              bool store, Put& put) {
+  FFSums r{{0.0f, 0.0f}, {0.0f, 0.0f}, {1.0f, 0.0f}};
   FF carry{1.0f, 0.0f};
-  for (int64_t base = m + 1; base <= R; base += 32 * kRun) {
-    const int64_t k0 = base + (int64_t)lane * kRun;
-    FF loc[kRun], pr{1.0f, 0.0f};
+  if (dir == 0) {
+    const FF xf = ff_from(x);
+    for (int64_t base = m + 1; base <= R; base += 32 * kRun) {
+      const int64_t k0 = base + (int64_t)lane * kRun;
+      FF loc[kRun], pr{1.0f, 0.0f};
 #pragma unroll
-    for (int b = 0; b < kRun; ++b) {
-      const int64_t k = k0 + b;
-      const FF term = k <= R ? ff_mul(xf, ff_rcp_int((float)k)) : FF{1.0f, 0.0f};
-      pr = ff_mul(pr, term);
-      loc[b] = pr;
-    }
-    const FF incl = ff_warp_incl_prod(pr, lane);
-    FF excl = ff_shfl_up(incl, 1);
-    if (lane == 0) excl = FF{1.0f, 0.0f};
-    const FF pre = ff_mul(carry, excl);
-#pragma unroll
-    for (int b = 0; b < kRun; ++b) {
-      const int64_t k = k0 + b;
-      if (k <= R) {
-        const FF w = ff_mul(pre, loc[b]);
-        sw = ff_add(sw, w);
-        if (k > K) st = ff_add(st, w);
-        else if (store) put(k, w);
+      for (int b = 0; b < kRun; ++b) {
+        const int64_t k = k0 + b;
+        const FF term = k <= R ? ff_mul(xf, ff_rcp_int((float)k)) : FF{1.0f, 0.0f};
+        pr = ff_mul(pr, term);
+        loc[b] = pr;
       }
-    }
-    const FF last = ff_mul(pre, pr);
-    carry = FF{__shfl_sync(kFull, last.hi, 31), __shfl_sync(kFull, last.lo, 31)};
-  }
-  carry = FF{1.0f, 0.0f};
-  for (int64_t base = m - 1; base >= L; base -= 32 * kRun) {
-    const int64_t k0 = base - (int64_t)lane * kRun;
-    FF loc[kRun], pr{1.0f, 0.0f};
+      const FF incl = ff_warp_incl_prod(pr, lane);
+      FF excl = ff_shfl_up(incl, 1);
+      if (lane == 0) excl = FF{1.0f, 0.0f};
+      const FF pre = ff_mul(carry, excl);
 #pragma unroll
-    for (int b = 0; b < kRun; ++b) {
-      const int64_t k = k0 - b;
-      const FF term = k >= L ? ff_mul_int(invx, (float)(k + 1)) : FF{1.0f, 0.0f};
-      pr = ff_mul(pr, term);
-      loc[b] = pr;
-    }
-    const FF incl = ff_warp_incl_prod(pr, lane);
-    FF excl = ff_shfl_up(incl, 1);
-    if (lane == 0) excl = FF{1.0f, 0.0f};
-    const FF pre = ff_mul(carry, excl);
-#pragma unroll
-    for (int b = 0; b < kRun; ++b) {
-      const int64_t k = k0 - b;
-      if (k >= L) {
-        const FF w = ff_mul(pre, loc[b]);
-        sw = ff_add(sw, w);
-        if (store) put(k, w);
-        if (k == L) wl = w;
+      for (int b = 0; b < kRun; ++b) {
+        const int64_t k = k0 + b;
+        if (k <= R) {
+          const FF w = ff_mul(pre, loc[b]);
+          r.all = ff_add(r.all, w);
+          if (k > K) r.tail = ff_add(r.tail, w);
+          else if (store) put(k, w);
+        }
       }
+      const FF last = ff_mul(pre, pr);
+      carry = FF{__shfl_sync(kFull, last.hi, 31), __shfl_sync(kFull, last.lo, 31)};
     }
-    const FF last = ff_mul(pre, pr);
-    carry = FF{__shfl_sync(kFull, last.hi, 31), __shfl_sync(kFull, last.lo, 31)};
+  } else {
+    const FF invx = ff_from(invxd);
+    for (int64_t base = m - 1; base >= L; base -= 32 * kRun) {
+      const int64_t k0 = base - (int64_t)lane * kRun;
+      FF loc[kRun], pr{1.0f, 0.0f}, wl{0.0f, 0.0f};
+#pragma unroll
+      for (int b = 0; b < kRun; ++b) {
+        const int64_t k = k0 - b;
+        const FF term = k >= L ? ff_mul_int(invx, (float)(k + 1)) : FF{1.0f, 0.0f};
+        pr = ff_mul(pr, term);
+        loc[b] = pr;
+      }
+      const FF incl = ff_warp_incl_prod(pr, lane);
+      FF excl = ff_shfl_up(incl, 1);
+      if (lane == 0) excl = FF{1.0f, 0.0f};
+      const FF pre = ff_mul(carry, excl);
+#pragma unroll
+      for (int b = 0; b < kRun; ++b) {
+        const int64_t k = k0 - b;
+        if (k >= L) {
+          const FF w = ff_mul(pre, loc[b]);
+          r.all = ff_add(r.all, w);
+          if (store) put(k, w);
+          if (k == L) wl = w;
+        }
+      }
+      if (base - L < 32 * kRun) {  // the run that holds L
+        const int src = (int)((base - L) / kRun);
+        r.wL = FF{__shfl_sync(kFull, wl.hi, src), __shfl_sync(kFull, wl.lo, src)};
+      }
+      const FF last = ff_mul(pre, pr);
+      carry = FF{__shfl_sync(kFull, last.hi, 31), __shfl_sync(kFull, last.lo, 31)};
+    }
   }
-  W = warp_sum(ff_to(sw));
-  tailsum = warp_sum(ff_to(st));
-  wL = (L == m) ? 1.0 : warp_sum(ff_to(wl));  // w_L sits in exactly one lane
+  r.all = ff_warp_sum(r.all);
+  r.tail = ff_warp_sum(r.tail);
+  return r;
 }
 
-// The same in FP64 (x / k as x times the reciprocal of k), for the FP64
-// chains, whose 1e-12 agreement with the oracle needs weights (and P_L, the
-// start of the recurrence of a window without a stored copy) to FP64
-// precision.
+// The same in FP64, for the FP64 chains, whose 1e-12 agreement with the oracle
+// needs weights (and P_L, the start of the recurrence of a window without a
+// stored copy) to FP64 precision.  Upward, x^b / (k0 (k0+1) ..) for the run's
+// positions b comes from one reciprocal of the product of all its k, multiplied
+// back from the run's end (products of 8 factors up to 2^40 stay finite).
+struct Sums64 {
+  double all, tail, wL;
+};
 template <class Put>
-__device__ void paper_weights64(double x, int64_t L, int64_t K, int64_t m, int64_t R, int lane, bool store,
-                              Put& put, double& W, double& tailsum, double& wL) {
-  double sw = lane == 0 ? 1.0 : 0.0, st = 0.0, wl = 0.0;
-  if (store && lane == 0) put(m, 1.0);
+__device__ Sums64 dir_weights64(int dir, double x, double invx, int64_t L, int64_t K, int64_t m, int64_t R, int lane,
+                                bool store, Put& put) {
+  Sums64 r{0.0, 0.0, 1.0};
   double carry = 1.0;
-  for (int64_t base = m + 1; base <= R; base += 32 * kRun) {
-    const int64_t k0 = base + (int64_t)lane * kRun;
-    double loc[kRun], pr = 1.0;
+  double xp[kRun];  // x^(b+1), or x^-(b+1)
+  xp[0] = dir == 0 ? x : invx;
 #pragma unroll
-    for (int b = 0; b < kRun; ++b) {
-      const int64_t k = k0 + b;
-      const double term = k <= R ? __dmul_rn(x, __drcp_rn((double)k)) : 1.0;
-      pr = __dmul_rn(pr, term);
-      loc[b] = pr;
-    }
-    const double incl = warp_incl_prod(pr, lane);
-    double excl = __shfl_up_sync(kFull, incl, 1);
-    if (lane == 0) excl = 1.0;
-    const double pre = __dmul_rn(carry, excl);
+  for (int b = 1; b < kRun; ++b) xp[b] = __dmul_rn(xp[b - 1], xp[0]);
+  if (dir == 0) {
+    for (int64_t base = m + 1; base <= R; base += 32 * kRun) {
+      const int64_t k0 = base + (int64_t)lane * kRun;
+      const double kd = (double)k0;
+      double loc[kRun], pk = kd;
 #pragma unroll
-    for (int b = 0; b < kRun; ++b) {
-      const int64_t k = k0 + b;
-      if (k <= R) {
-        const double w = __dmul_rn(pre, loc[b]);
-        sw += w;
-        if (k > K) st += w;
-        else if (store) put(k, w);
+      for (int b = 1; b < kRun; ++b) pk = __dmul_rn(pk, kd + (double)b);
+      double inv = __drcp_rn(pk);  // 1 / (k0 .. k0 + 7)
+#pragma unroll
+      for (int b = kRun - 1; b >= 0; --b) {
+        loc[b] = __dmul_rn(xp[b], inv);
+        inv = __dmul_rn(inv, kd + (double)b);
       }
-    }
-    carry = __shfl_sync(kFull, __dmul_rn(pre, pr), 31);
-  }
-  const double invx = __drcp_rn(x);
-  carry = 1.0;
-  for (int64_t base = m - 1; base >= L; base -= 32 * kRun) {
-    const int64_t k0 = base - (int64_t)lane * kRun;
-    double loc[kRun], pr = 1.0;
+      const double incl = warp_incl_prod(loc[kRun - 1], lane);
+      double excl = __shfl_up_sync(kFull, incl, 1);
+      if (lane == 0) excl = 1.0;
+      const double pre = __dmul_rn(carry, excl);
 #pragma unroll
-    for (int b = 0; b < kRun; ++b) {
-      const int64_t k = k0 - b;
-      const double term = k >= L ? __dmul_rn((double)(k + 1), invx) : 1.0;
-      pr = __dmul_rn(pr, term);
-      loc[b] = pr;
-    }
-    const double incl = warp_incl_prod(pr, lane);
-    double excl = __shfl_up_sync(kFull, incl, 1);
-    if (lane == 0) excl = 1.0;
-    const double pre = __dmul_rn(carry, excl);
-#pragma unroll
-    for (int b = 0; b < kRun; ++b) {
-      const int64_t k = k0 - b;
-      if (k >= L) {
-        const double w = __dmul_rn(pre, loc[b]);
-        sw += w;
-        if (store) put(k, w);
-        if (k == L) wl = w;
+      for (int b = 0; b < kRun; ++b) {
+        const int64_t k = k0 + b;
+        if (k <= R) {
+          const double w = __dmul_rn(pre, loc[b]);
+          r.all += w;
+          if (k > K) r.tail += w;
+          else if (store) put(k, w);
+        }
       }
+      carry = __dmul_rn(carry, __shfl_sync(kFull, incl, 31));
     }
-    carry = __shfl_sync(kFull, __dmul_rn(pre, pr), 31);
+  } else {
+    for (int64_t base = m - 1; base >= L; base -= 32 * kRun) {
+      const int64_t k0 = base - (int64_t)lane * kRun;
+      const double kd = (double)(k0 + 1);
+      double loc[kRun], pk = 1.0, wl = 0.0;
+#pragma unroll
+      for (int b = 0; b < kRun; ++b) {
+        // (Below L the products only feed lanes that hold no weight; below 0
+        // the factors are taken as 1 so that they stay finite and positive.)
+        pk = __dmul_rn(pk, k0 - b >= L ? kd - (double)b : 1.0);
+        loc[b] = __dmul_rn(pk, xp[b]);
+      }
+      const double incl = warp_incl_prod(loc[kRun - 1], lane);
+      double excl = __shfl_up_sync(kFull, incl, 1);
+      if (lane == 0) excl = 1.0;
+      const double pre = __dmul_rn(carry, excl);
+#pragma unroll
+      for (int b = 0; b < kRun; ++b) {
+        const int64_t k = k0 - b;
+        if (k >= L) {
+          const double w = __dmul_rn(pre, loc[b]);
+          r.all += w;
+          if (store) put(k, w);
+          if (k == L) wl = w;
+        }
+      }
+      if (base - L < 32 * kRun) r.wL = __shfl_sync(kFull, wl, (int)((base - L) / kRun));
+      carry = __dmul_rn(carry, __shfl_sync(kFull, incl, 31));
+    }
   }
-  W = warp_sum(sw);
-  tailsum = warp_sum(st);
-  wL = (L == m) ? 1.0 : warp_sum(wl);  // w_L sits in exactly one lane
+  r.all = warp_sum(r.all);
+  r.tail = warp_sum(r.tail);
+  return r;
 }
 
-// Plan one time on one warp.  doff: the arena offset reserved for this
-// window's weights (paper's rule), or -1.
-__device__ void plan_time(const PlanParams& p, double omega, double t, Win* dst, int lane, long long doff_in) {
+// Plan one time on one warp (tolerance rule).
+__device__ void plan_time(const PlanParams& p, double omega, double t, Win* dst, int lane) {
   Win r;
   double x = __dmul_rn(omega, t);
   r.x = x;
   if (x == 0.0) {  // t = 0 or no transitions: rho*(t) = rho0
     r.L = 0;
-    r.K = (p.trunc_mode == MJP_TRUNC_PAPER) ? 1 : 0;
+    r.K = 0;
     r.PL = 1.0;
     r.tail = 0.0;
     r.woff = -1;
     if (lane == 0) *dst = r;
     return;
   }
-  double s = __dsqrt_rn(x);
-  double kstar = __dadd_rn(x, __dmul_rn(6.0, s));  // Omega t + 6 sqrt(Omega t)
-  if (!(kstar + 1.0 <= (double)p.kcap)) {  // also catches inf/NaN; nothing loops
+  int64_t K = 0, L = 0;
+  if (!window_bounds(p, x, L, K)) {  // K above the cap (also inf / NaN; nothing loops)
     if (lane == 0) {
       set_status(p.status, kStatusKcap);
-      // A NaN weight makes this time's result (and a log-likelihood using it)
-      // NaN, so a caller that keeps going (a sampler) rejects the parameters.
-      r.L = 0; r.K = 0; r.PL = __longlong_as_double(0x7ff8000000000000LL); r.tail = 0.0; r.woff = -1;
-      *dst = r;
+      *dst = capped_window(x);
     }
     return;
   }
-  int64_t K = 0, L = 0;
-  window_bounds(p, x, L, K);
+  const double s = __dsqrt_rn(x);
   int64_t m = (int64_t)floor(x);
   int64_t R = (int64_t)floor(x + 10.0 * s) + 10;
-
-  // Under the paper's rule K is known before the scans: the window [L, K]
-  // of the weight arena was reserved by the CTA and receives the
-  // unnormalised weights as the scans form them (scaled by 1 / W below), so
-  // no second pair of scans is needed.
-  const bool direct = p.arena && p.trunc_mode == MJP_TRUNC_PAPER;
-  const int64_t dsize = K - L + 1;
-  const unsigned long long doff = doff_in >= 0 ? (unsigned long long)doff_in : 0ull;
-  const bool dstore = direct && doff_in >= 0;
-  // Raw weights: float-float for FP32 chains, FP64 for FP64 chains (whose
-  // arena holds doubles).
-  auto put_raw = [&](int64_t k, FF w) { reinterpret_cast<float*>(p.arena)[doff + (k - L)] = w.hi; };
-  auto put_raw64 = [&](int64_t k, double w) {
-    if (p.arena_fp64) reinterpret_cast<double*>(p.arena)[doff + (k - L)] = w;
-    else reinterpret_cast<float*>(p.arena)[doff + (k - L)] = (float)w;
-  };
-  if (p.trunc_mode == MJP_TRUNC_PAPER) {
-    double W, ts, wL;
-    if (p.fp64_weights || p.arena_fp64) paper_weights64(x, L, K, m, R, lane, dstore, put_raw64, W, ts, wL);
-    else paper_weights(x, L, K, m, R, lane, dstore, put_raw, W, ts, wL);
-    r.L = L;
-    r.K = K;
-    r.PL = wL / W;
-    r.tail = ts / W;
-    r.woff = -1;
-    if (dstore) {
-      r.woff = (int64_t)doff;
-      __syncwarp();  // every lane's raw weights are visible to the lane that scales them
-      const double invW = __ddiv_rn(1.0, W);
-      if (p.arena_fp64) {
-        double* a = reinterpret_cast<double*>(p.arena) + doff;
-        for (int64_t j = lane; j < dsize; j += 32) {
-          double v = __dmul_rn(a[j], invW);
-          if (L + j == K) v = v + r.tail;
-          a[j] = v;
-        }
-      } else {  // FP32 weights scaled in float-float on the FP32 pipe
-        float* a = reinterpret_cast<float*>(p.arena) + doff;
-        const FF invWf = ff_from(invW);
-        for (int64_t j = lane; j < dsize; j += 32) {
-          FF v = ff_mul(FF{a[j], 0.0f}, invWf);
-          if (L + j == K) v = ff_add(v, ff_from(r.tail));
-          a[j] = __fadd_rn(v.hi, v.lo);
-        }
-      }
-    }
-    if (lane == 0) *dst = r;
-    return;
-  }
 
   // Tolerance rule.  Upward from the mode: w_k = w_{k-1} x / k, w_m = 1.
   Kahan sum;
@@ -504,10 +507,20 @@ __device__ void plan_time(const PlanParams& p, double omega, double t, Win* dst,
   if (lane == 0) *dst = r;
 }
 
+// max_n e_n over the corners of the box: the last and last but one state of
+// every axis, both gene states (thread c < 8).
+__device__ double corner_rate(const PlanParams& p, int64_t M, int64_t N, int c, const double* th) {
+  const int64_t m = M - 1 - (c & 1);
+  if (p.kind == MJP_BD1D) return c < 2 && m >= 0 ? exit_rate(p.kind, M, 1, m, th) : 0.0;
+  if (p.kind == MJP_TWOSTATE) return c < 4 ? exit_rate(p.kind, M, 2, m + (c >> 1) * M, th) : 0.0;
+  const int64_t rows = p.kind == MJP_AUTOREG ? p.P / 2 : p.P, q = rows - 1 - ((c >> 1) & 1);
+  if (m < 0 || q < 0 || (p.kind != MJP_AUTOREG && c >= 4)) return 0.0;
+  return exit_rate(p.kind, M, p.P, m + M * q + M * rows * (c >> 2), th);
+}
+
 __global__ void __launch_bounds__(256) plan_kernel(PlanParams p) {
   const int job = blockIdx.x;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  __shared__ double red[8];
   __shared__ double s_omega;
   double omega;
   if (p.omega_fixed >= 0.0) {
@@ -515,62 +528,190 @@ __global__ void __launch_bounds__(256) plan_kernel(PlanParams p) {
   } else {
     const double* th = p.theta + (int64_t)job * p.ntheta;
     const int64_t NJ = p.jobN ? (int64_t)p.jobN[job] : p.N;
-    const int64_t MJ = p.jobN ? NJ : p.M;
-    double mx = 0.0;
-    for (int64_t n = tid; n < NJ; n += blockDim.x) {
-      double e = exit_rate(p.kind, MJ, p.P, n, th);
-      mx = e > mx ? e : mx;
-    }
+    if (warp == 0) {
+      double mx = lane < 8 ? corner_rate(p, p.jobN ? NJ : p.M, NJ, lane, th) : 0.0;
+      if (!(mx > 0.0)) mx = 0.0;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      double t = __shfl_xor_sync(kFull, mx, o);
-      mx = t > mx ? t : mx;
-    }
-    if (lane == 0) red[warp] = mx;
-    __syncthreads();
-    if (tid == 0) {
-      double v = 0.0;
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v = red[w] > v ? red[w] : v;
-      s_omega = (v > 0.0) ? __dmul_rn(p.omega_factor, v) : 0.0;
+      for (int o = 4; o > 0; o >>= 1) {
+        const double t = __shfl_xor_sync(kFull, mx, o);
+        mx = t > mx ? t : mx;
+      }
+      if (lane == 0) s_omega = mx > 0.0 ? __dmul_rn(p.omega_factor, mx) : 0.0;
     }
     __syncthreads();
     omega = s_omega;
   }
   Win* wj = p.win + (int64_t)job * p.ntimes;
   const double* tj = p.times + (p.times_per_job ? (int64_t)job * p.ntimes : 0);
-  // Paper's rule: the weight windows of all this instance's times are
-  // reserved in one piece, in time order (the same layout every call, and an
-  // instance's windows either all fit or all run the chain's recurrence).
-  __shared__ long long s_off[kMaxTimes];
-  const bool direct = p.arena && p.trunc_mode == MJP_TRUNC_PAPER;
-  if (direct) {
-    for (int i = tid; i < p.ntimes; i += blockDim.x) {
-      int64_t L = 0, K = 0;
-      s_off[i] = window_bounds(p, __dmul_rn(omega, tj[i]), L, K) ? (long long)(K - L + 1) : 0;
-    }
+  const int nt = p.ntimes;
+  if (p.trunc_mode != MJP_TRUNC_PAPER) {
+    for (int i = warp; i < nt; i += blockDim.x >> 5) plan_time(p, omega, tj[i], wj + i, lane);
     __syncthreads();
     if (tid == 0) {
-      long long tot = 0;
-      for (int i = 0; i < p.ntimes; ++i) {
-        const long long sz = s_off[i];
-        s_off[i] = sz > 0 ? tot : -1;
-        tot += sz;
-      }
-      const unsigned long long base = tot > 0 ? atomicAdd(p.arena_used, (unsigned long long)tot) : 0ull;
-      const bool fit = (long long)base + tot <= (long long)p.arena_cap;
-      for (int i = 0; i < p.ntimes; ++i) s_off[i] = (fit && s_off[i] >= 0) ? (long long)base + s_off[i] : -1;
-      if (!fit && p.arena_over) atomicOr(p.arena_over, 1);
+      int64_t kmax = 0;
+      for (int i = 0; i < nt; ++i) kmax = wj[i].K > kmax ? wj[i].K : kmax;
+      p.info[job].omega = omega;
+      p.info[job].Kmax = kmax;
     }
-    __syncthreads();
+    return;
   }
-  for (int i = warp; i < p.ntimes; i += blockDim.x >> 5)
-    plan_time(p, omega, tj[i], wj + i, lane, direct ? s_off[i] : -1);
+
+  // ---- windows: a thread each ------------------------------------------------
+  // s_kind: 0 = a window, 1 = no chain (x = 0), 2 = K above the cap.
+  __shared__ double s_x[kMaxTimes], s_invx[kMaxTimes];
+  __shared__ long long s_L[kMaxTimes], s_K[kMaxTimes], s_R[kMaxTimes], s_off[kMaxTimes];
+  __shared__ signed char s_kind[kMaxTimes];
+  // Sums of both directions, then W in [0] and its reciprocal in [1].
+  __shared__ double s_sum[kMaxTimes][2], s_tail[kMaxTimes], s_wL[kMaxTimes];
+  __shared__ long long s_tot;
+  static_assert(kMaxTimes <= 256, "a thread per window");
+  const bool fp64 = p.fp64_weights || p.arena_fp64;
+  if (tid < nt) {
+    const double x = __dmul_rn(omega, tj[tid]);
+    int64_t L = 0, K = 0;
+    long long size = 0;
+    signed char kind = x == 0.0 ? 1 : 2;
+    s_x[tid] = x;
+    if (window_bounds(p, x, L, K)) {
+      kind = 0;
+      s_R[tid] = (int64_t)floor(x + 10.0 * __dsqrt_rn(x)) + 10;
+      s_invx[tid] = fp64 ? __drcp_rn(x) : 1.0 / x;
+      size = K - L + 1;
+    } else if (kind == 1) {
+      K = 1;
+    }
+    s_L[tid] = L;
+    s_K[tid] = K;
+    s_kind[tid] = kind;
+    s_off[tid] = size;
+  }
   __syncthreads();
-  if (tid == 0) {
-    int64_t kmax = 0;
-    for (int i = 0; i < p.ntimes; ++i) kmax = wj[i].K > kmax ? wj[i].K : kmax;
-    p.info[job].omega = omega;
-    p.info[job].Kmax = kmax;
+  // The windows of all this instance's times are reserved in one piece, in time
+  // order (the same layout every call, and an instance's windows either all fit
+  // or all run the chain's recurrence); a single instance starts at 0.
+  if (warp == 0) {
+    long long tot = 0, kmax = 0;
+    for (int i0 = 0; i0 < nt; i0 += 32) {
+      const int i = i0 + lane;
+      const long long sz = i < nt ? s_off[i] : 0;
+      long long incl = sz;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const long long t = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += t;
+      }
+      if (i < nt) s_off[i] = sz > 0 ? tot + incl - sz : -1;
+      tot += __shfl_sync(kFull, incl, 31);
+      const long long k = i < nt ? s_K[i] : 0;
+      kmax = k > kmax ? k : kmax;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const long long t = __shfl_xor_sync(kFull, kmax, o);
+      kmax = t > kmax ? t : kmax;
+    }
+    if (lane == 0) {
+      long long base = -1;  // no place
+      if (p.arena) {
+        base = p.B > 1 && tot > 0 ? (long long)atomicAdd(p.arena_used, (unsigned long long)tot) : 0;
+        if (base + tot > (long long)p.arena_cap) {
+          base = -1;
+          if (p.arena_over) atomicOr(p.arena_over, 1);
+        }
+      }
+      s_tot = base;
+      if (blockIdx.y == 0) {
+        p.info[job].omega = omega;
+        p.info[job].Kmax = kmax;
+      }
+    }
+  }
+  __syncthreads();
+  const long long abase = s_tot;
+  const bool place = abase >= 0;
+
+  // ---- weights: a warp per window and direction --------------------------------
+  const int i0 = blockIdx.y, step = gridDim.y;  // this CTA's windows: i0, i0 + step, ...
+  const int nw = i0 < nt ? (nt - i0 + step - 1) / step : 0;
+  for (int q = warp; q < 2 * nw; q += blockDim.x >> 5) {
+    const int i = i0 + (q >> 1) * step, dir = q & 1;
+    if (s_kind[i] != 0) continue;
+    const double x = s_x[i];
+    const int64_t L = s_L[i], K = s_K[i], m = (int64_t)floor(x), R = s_R[i];
+    const long long off = abase + s_off[i] - L;
+    const bool mode = dir == 0 && lane == 0 && place;  // the mode's own weight
+    if (fp64) {
+      auto put = [&](int64_t k, double w) {
+        if (p.arena_fp64) reinterpret_cast<double*>(p.arena)[off + k] = w;
+        else reinterpret_cast<float*>(p.arena)[off + k] = (float)w;
+      };
+      if (mode) put(m, 1.0);
+      const Sums64 r = dir_weights64(dir, x, s_invx[i], L, K, m, R, lane, place, put);
+      if (lane == 0) {
+        s_sum[i][dir] = r.all;
+        if (dir == 0) s_tail[i] = r.tail;
+        else s_wL[i] = r.wL;
+      }
+    } else {
+      auto put = [&](int64_t k, FF w) { reinterpret_cast<float*>(p.arena)[off + k] = w.hi; };
+      if (mode) put(m, FF{1.0f, 0.0f});
+      const FFSums r = dir_weights(dir, x, s_invx[i], L, K, m, R, lane, place, put);
+      if (lane == 0) {
+        s_sum[i][dir] = ff_to(r.all);
+        if (dir == 0) s_tail[i] = ff_to(r.tail);
+        else s_wL[i] = ff_to(r.wL);
+      }
+    }
+  }
+  __syncthreads();
+
+  // ---- normalisation: a thread per window ---------------------------------------
+  if (tid < nt && tid % step == i0) {
+    Win r;
+    if (s_kind[tid] == 2) {
+      set_status(p.status, kStatusKcap);
+      r = capped_window(s_x[tid]);
+    } else {
+      r.x = s_x[tid];
+      r.L = s_L[tid];
+      r.K = s_K[tid];
+      r.PL = 1.0;
+      r.tail = 0.0;
+      r.woff = -1;
+      if (s_kind[tid] == 0) {
+        const double invW = __ddiv_rn(1.0, 1.0 + s_sum[tid][0] + s_sum[tid][1]);
+        r.PL = __dmul_rn(s_wL[tid], invW);
+        r.tail = __dmul_rn(s_tail[tid], invW);
+        if (place) r.woff = abase + s_off[tid];
+        s_tail[tid] = r.tail;
+        s_sum[tid][1] = invW;
+      }
+    }
+    wj[tid] = r;
+  }
+  __syncthreads();  // every raw weight and every factor is visible to the warps that scale them
+  if (!place) return;
+  for (int q = warp; q < nw; q += blockDim.x >> 5) {
+    const int i = i0 + q * step;
+    if (s_kind[i] != 0) continue;
+    const int64_t size = s_K[i] - s_L[i] + 1;
+    const double invW = s_sum[i][1], tail = s_tail[i];
+    if (p.arena_fp64) {
+      double* a = reinterpret_cast<double*>(p.arena) + abase + s_off[i];
+      for (int64_t j = lane; j < size; j += 32) {
+        double v = __dmul_rn(a[j], invW);
+        if (j == size - 1) v = v + tail;
+        a[j] = v;
+      }
+    } else {  // FP32 weights scaled in float-float on the FP32 pipe
+      float* a = reinterpret_cast<float*>(p.arena) + abase + s_off[i];
+      const FF invWf = ff_from(invW);
+      for (int64_t j = lane; j < size; j += 32) {
+        FF v = ff_mul(FF{a[j], 0.0f}, invWf);
+        if (j == size - 1) v = ff_add(v, ff_from(tail));
+        a[j] = __fadd_rn(v.hi, v.lo);
+      }
+    }
   }
 }
 
@@ -594,7 +735,9 @@ __global__ void order_jobs_kernel(const JobInfo* info, int B, int32_t* map) {
 
 cudaError_t launch_plan(const PlanParams& p, cudaStream_t s) {
   if (p.B <= 0) return cudaSuccess;
-  plan_kernel<<<p.B, 256, 0, s>>>(p);
+  // A single instance by the paper's rule: a CTA per window.
+  const int split = p.B == 1 && p.trunc_mode == MJP_TRUNC_PAPER ? (p.ntimes < 64 ? p.ntimes : 64) : 1;
+  plan_kernel<<<dim3((unsigned)p.B, (unsigned)split), 256, 0, s>>>(p);
   return cudaGetLastError();
 }
 
