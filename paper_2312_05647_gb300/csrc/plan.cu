@@ -22,8 +22,8 @@
 // lanes of a warp did alike (roots and divisions, about 250 instructions per
 // window) runs a thread per window instead, and the FP64 reciprocals of 8
 // consecutive k are one reciprocal of their product and 8 multiplications.
-// Measured: 256 thetas x 50 times FP32 151 -> 117 us, 10^4 thetas x 5 times
-// FP64 756 -> 567 us, one theta x 5 times FP64 20 -> 12 us.
+// Measured: 256 thetas x 50 times FP32 151 -> 108 us, 10^4 thetas x 5 times
+// FP64 756 -> 543 us, one theta x 5 times FP64 20 -> 12 us.
 //
 // Tolerance rule: a warp per window does everything (K is known only after the
 // scans).
@@ -213,19 +213,19 @@ __device__ __forceinline__ FF ff_warp_sum(FF v) {
     v = ff_add(v, FF{__shfl_xor_sync(kFull, v.hi, o), __shfl_xor_sync(kFull, v.lo, o)});
   return v;
 }
-template <class Put>
-__device__ FFSums dir_weights(int dir, double x, double invxd, int64_t L, int64_t K, int64_t m, int64_t R, int lane,
-                              bool store, Put& put) {
+// I: 32-bit jump counts where they fit (a 64-bit integer's conversion to FP32
+// runs at the FP64 pipe's rate, one per weight).
+template <class I, class Put>
+__device__ FFSums dir_weights(int dir, FF xf, FF invx, I L, I K, I m, I R, int lane, bool store, Put& put) {
   FFSums r{{0.0f, 0.0f}, {0.0f, 0.0f}, {1.0f, 0.0f}};
   FF carry{1.0f, 0.0f};
   if (dir == 0) {
-    const FF xf = ff_from(x);
-    for (int64_t base = m + 1; base <= R; base += 32 * kRun) {
-      const int64_t k0 = base + (int64_t)lane * kRun;
+    for (I base = m + 1; base <= R; base += 32 * kRun) {
+      const I k0 = base + lane * kRun;
       FF loc[kRun], pr{1.0f, 0.0f};
 #pragma unroll
       for (int b = 0; b < kRun; ++b) {
-        const int64_t k = k0 + b;
+        const I k = k0 + b;
         const FF term = k <= R ? ff_mul(xf, ff_rcp_int((float)k)) : FF{1.0f, 0.0f};
         pr = ff_mul(pr, term);
         loc[b] = pr;
@@ -236,7 +236,7 @@ __device__ FFSums dir_weights(int dir, double x, double invxd, int64_t L, int64_
       const FF pre = ff_mul(carry, excl);
 #pragma unroll
       for (int b = 0; b < kRun; ++b) {
-        const int64_t k = k0 + b;
+        const I k = k0 + b;
         if (k <= R) {
           const FF w = ff_mul(pre, loc[b]);
           r.all = ff_add(r.all, w);
@@ -248,13 +248,12 @@ __device__ FFSums dir_weights(int dir, double x, double invxd, int64_t L, int64_
       carry = FF{__shfl_sync(kFull, last.hi, 31), __shfl_sync(kFull, last.lo, 31)};
     }
   } else {
-    const FF invx = ff_from(invxd);
-    for (int64_t base = m - 1; base >= L; base -= 32 * kRun) {
-      const int64_t k0 = base - (int64_t)lane * kRun;
+    for (I base = m - 1; base >= L; base -= 32 * kRun) {
+      const I k0 = base - lane * kRun;
       FF loc[kRun], pr{1.0f, 0.0f}, wl{0.0f, 0.0f};
 #pragma unroll
       for (int b = 0; b < kRun; ++b) {
-        const int64_t k = k0 - b;
+        const I k = k0 - b;
         const FF term = k >= L ? ff_mul_int(invx, (float)(k + 1)) : FF{1.0f, 0.0f};
         pr = ff_mul(pr, term);
         loc[b] = pr;
@@ -265,7 +264,7 @@ __device__ FFSums dir_weights(int dir, double x, double invxd, int64_t L, int64_
       const FF pre = ff_mul(carry, excl);
 #pragma unroll
       for (int b = 0; b < kRun; ++b) {
-        const int64_t k = k0 - b;
+        const I k = k0 - b;
         if (k >= L) {
           const FF w = ff_mul(pre, loc[b]);
           r.all = ff_add(r.all, w);
@@ -282,7 +281,7 @@ __device__ FFSums dir_weights(int dir, double x, double invxd, int64_t L, int64_
     }
   }
   r.all = ff_warp_sum(r.all);
-  r.tail = ff_warp_sum(r.tail);
+  if (dir == 0) r.tail = ff_warp_sum(r.tail);
   return r;
 }
 
@@ -320,16 +319,18 @@ __device__ Sums64 dir_weights64(int dir, double x, double invx, int64_t L, int64
       double excl = __shfl_up_sync(kFull, incl, 1);
       if (lane == 0) excl = 1.0;
       const double pre = __dmul_rn(carry, excl);
+      // The run's sum from its far end: at k = K + 1 it holds the run's tail.
+      double run = 0.0, rest = 0.0;
 #pragma unroll
-      for (int b = 0; b < kRun; ++b) {
+      for (int b = kRun - 1; b >= 0; --b) {
         const int64_t k = k0 + b;
-        if (k <= R) {
-          const double w = __dmul_rn(pre, loc[b]);
-          r.all += w;
-          if (k > K) r.tail += w;
-          else if (store) put(k, w);
-        }
+        const double w = __dmul_rn(pre, loc[b]);
+        if (k <= R) run += w;
+        if (k > K) rest = run;
+        else if (store && k <= R) put(k, w);
       }
+      r.all += run;
+      r.tail += rest;
       carry = __dmul_rn(carry, __shfl_sync(kFull, incl, 31));
     }
   } else {
@@ -363,7 +364,7 @@ __device__ Sums64 dir_weights64(int dir, double x, double invx, int64_t L, int64
     }
   }
   r.all = warp_sum(r.all);
-  r.tail = warp_sum(r.tail);
+  if (dir == 0) r.tail = warp_sum(r.tail);
   return r;
 }
 
@@ -561,8 +562,12 @@ __global__ void __launch_bounds__(256) plan_kernel(PlanParams p) {
   __shared__ double s_x[kMaxTimes], s_invx[kMaxTimes];
   __shared__ long long s_L[kMaxTimes], s_K[kMaxTimes], s_R[kMaxTimes], s_off[kMaxTimes];
   __shared__ signed char s_kind[kMaxTimes];
-  // Sums of both directions, then W in [0] and its reciprocal in [1].
+  // Sums of both directions, the tail and w_L (FP32 chains: as float-float in
+  // the same place), later 1 / W in s_sum[.][1]; x and 1 / x in float-float.
   __shared__ double s_sum[kMaxTimes][2], s_tail[kMaxTimes], s_wL[kMaxTimes];
+  __shared__ FF s_xf[kMaxTimes], s_invxf[kMaxTimes];
+  static_assert(sizeof(FF) == sizeof(double), "float-float sums share the doubles' place");
+  auto ff_at = [](double& d) -> FF& { return reinterpret_cast<FF&>(d); };
   __shared__ long long s_tot;
   static_assert(kMaxTimes <= 256, "a thread per window");
   const bool fp64 = p.fp64_weights || p.arena_fp64;
@@ -576,6 +581,10 @@ __global__ void __launch_bounds__(256) plan_kernel(PlanParams p) {
       kind = 0;
       s_R[tid] = (int64_t)floor(x + 10.0 * __dsqrt_rn(x)) + 10;
       s_invx[tid] = fp64 ? __drcp_rn(x) : 1.0 / x;
+      if (!fp64) {
+        s_xf[tid] = ff_from(x);
+        s_invxf[tid] = ff_from(s_invx[tid]);
+      }
       size = K - L + 1;
     } else if (kind == 1) {
       K = 1;
@@ -655,11 +664,13 @@ __global__ void __launch_bounds__(256) plan_kernel(PlanParams p) {
     } else {
       auto put = [&](int64_t k, FF w) { reinterpret_cast<float*>(p.arena)[off + k] = w.hi; };
       if (mode) put(m, FF{1.0f, 0.0f});
-      const FFSums r = dir_weights(dir, x, s_invx[i], L, K, m, R, lane, place, put);
+      const FFSums r = R < (1LL << 30)
+                           ? dir_weights<int>(dir, s_xf[i], s_invxf[i], (int)L, (int)K, (int)m, (int)R, lane, place, put)
+                           : dir_weights<int64_t>(dir, s_xf[i], s_invxf[i], L, K, m, R, lane, place, put);
       if (lane == 0) {
-        s_sum[i][dir] = ff_to(r.all);
-        if (dir == 0) s_tail[i] = ff_to(r.tail);
-        else s_wL[i] = ff_to(r.wL);
+        ff_at(s_sum[i][dir]) = r.all;
+        if (dir == 0) ff_at(s_tail[i]) = r.tail;
+        else ff_at(s_wL[i]) = r.wL;
       }
     }
   }
@@ -679,12 +690,22 @@ __global__ void __launch_bounds__(256) plan_kernel(PlanParams p) {
       r.tail = 0.0;
       r.woff = -1;
       if (s_kind[tid] == 0) {
+        if (!fp64) {
+          s_sum[tid][0] = ff_to(ff_at(s_sum[tid][0]));
+          s_sum[tid][1] = ff_to(ff_at(s_sum[tid][1]));
+          s_tail[tid] = ff_to(ff_at(s_tail[tid]));
+          s_wL[tid] = ff_to(ff_at(s_wL[tid]));
+        }
         const double invW = __ddiv_rn(1.0, 1.0 + s_sum[tid][0] + s_sum[tid][1]);
         r.PL = __dmul_rn(s_wL[tid], invW);
         r.tail = __dmul_rn(s_tail[tid], invW);
         if (place) r.woff = abase + s_off[tid];
         s_tail[tid] = r.tail;
         s_sum[tid][1] = invW;
+        if (!fp64) {
+          s_xf[tid] = ff_from(invW);
+          s_invxf[tid] = ff_from(r.tail);
+        }
       }
     }
     wj[tid] = r;
@@ -695,8 +716,8 @@ __global__ void __launch_bounds__(256) plan_kernel(PlanParams p) {
     const int i = i0 + q * step;
     if (s_kind[i] != 0) continue;
     const int64_t size = s_K[i] - s_L[i] + 1;
-    const double invW = s_sum[i][1], tail = s_tail[i];
     if (p.arena_fp64) {
+      const double invW = s_sum[i][1], tail = s_tail[i];
       double* a = reinterpret_cast<double*>(p.arena) + abase + s_off[i];
       for (int64_t j = lane; j < size; j += 32) {
         double v = __dmul_rn(a[j], invW);
@@ -705,10 +726,10 @@ __global__ void __launch_bounds__(256) plan_kernel(PlanParams p) {
       }
     } else {  // FP32 weights scaled in float-float on the FP32 pipe
       float* a = reinterpret_cast<float*>(p.arena) + abase + s_off[i];
-      const FF invWf = ff_from(invW);
+      const FF invWf = s_xf[i];
       for (int64_t j = lane; j < size; j += 32) {
         FF v = ff_mul(FF{a[j], 0.0f}, invWf);
-        if (j == size - 1) v = ff_add(v, ff_from(tail));
+        if (j == size - 1) v = ff_add(v, s_invxf[i]);
         a[j] = __fadd_rn(v.hi, v.lo);
       }
     }
