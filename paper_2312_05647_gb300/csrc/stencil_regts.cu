@@ -16,8 +16,9 @@
 // j - 1 and j + 1 component by component (the whole update runs on FP32x2
 // pairs) and the two gene states of a column sit in the same slot of the two
 // rows.  Only a thread's first and last column need another thread's value:
-// shuffles inside a warp, a double-buffered shared-memory slot and a named
-// barrier of the chain warps between warps.  The pairs rotate through QP + 1
+// shuffles inside a warp, a double-buffered shared-memory slot (one 8-byte
+// store by both end lanes at once, no branch per lane) and a named barrier of
+// the chain warps between warps.  The pairs rotate through QP + 1
 // register slots (pair j of rho_k is written over pair j - 1 of rho_{k-1},
 // its last reader), so an in-place jump copies no register.
 //
@@ -30,10 +31,11 @@
 // Observations (warp specialised).  After every jump the chain threads whose
 // columns hold observed states write their states of rho_k into a history in
 // shared memory: a row per state, 32 jump columns, two halves of 16 filled in
-// turn.  Separate reducer warps take each half when it is full: every
+// turn (behind the chain's barrier: only the hand-over below needs the writes).  Separate reducer warps take each half when it is full: every
 // observation group whose window meets those 16 jumps gets the weighted sum
-// over them, sum_k w_{i,k} sum_{s in g} rho_k[s] (two FP32 FMA chains of at
-// most 8 terms), added to the group's accumulator with a Kahan step, while
+// over them, sum_k w_{i,k} sum_{s in g} rho_k[s] (an FP32x2 FMA chain of 8
+// terms: even and odd jumps; the weight ring holds 0 outside a window, so no
+// term is tested), added to the group's accumulator with a Kahan step, while
 // the chain warps fill the other half.  Two mbarriers per half hand it over
 // (full: the chain threads have written it; empty: the reducers have read
 // it); every wait on them is bounded (p.wait_limit polls, MJP_OPT_WAIT_LIMIT)
@@ -42,6 +44,13 @@
 // planner's arena 32 jumps at a time, one chunk ahead; a window without a
 // stored copy runs the recurrence P_k = P_{k-1} x / k from P_L (FP64) while
 // its chunk is staged.
+//
+// Bound: the issue slots of an SM's chain and reducer warps together with the
+// latency of one jump (shuffle, barrier, a dependent chain of packed FMAs).
+// Measured (300 x 2 states, 256 thetas, 50 times): per-term window tests, three
+// scalar edge stores in two branches and the history in front of the barrier
+// 1,238 us of chain; packed sums without tests, one edge store, the history
+// behind the barrier 1,105 us, log-likelihoods the same bits.
 #include <algorithm>
 #include <type_traits>
 
@@ -73,7 +82,7 @@ struct TsLayout {
 // Y.x, Y.y, component-major) and a zero row (an absent second member).
 __host__ __device__ inline size_t ts_hist(int nslot) { return (size_t)(4 * nslot + 1) * kHS; }
 
-// Shared memory of one CTA: edge slots [2 parities][Wc + 2][3] (chain warps
+// Shared memory of one CTA: edge slots [2 parities][Wc + 2][4] (chain warps
 // 0..Wc-1 in slots 1..Wc, zero slots 0 and Wc + 1 beyond the first and last),
 // window tables, the weight ring [time][kWStride], the groups (member offsets
 // in the history, time, Kahan sum and compensation), the history [state
@@ -81,7 +90,7 @@ __host__ __device__ inline size_t ts_hist(int nslot) { return (size_t)(4 * nslot
 __host__ __device__ inline TsLayout ts_layout(int Wc, int nslot, int nt, int G) {
   TsLayout s;
   size_t o = 0;
-  s.edge = o; o += align_up(4 * 2 * 3 * (size_t)(Wc + 2), 16);
+  s.edge = o; o += align_up(4 * 2 * 4 * (size_t)(Wc + 2), 16);
   s.tx = o; o += 8 * (size_t)nt;
   s.tPL = o; o += 8 * (size_t)nt;
   s.ttail = o; o += 8 * (size_t)nt;
@@ -172,7 +181,7 @@ __global__ void __launch_bounds__(32 * (kMaxChainWarps + kReduceWarps))
   const int job = p.job_map ? p.job_map[blockIdx.x] : (int)blockIdx.x;
   const int nt = p.ntimes, M = p.M, G = p.G;
   const TsLayout Ly = ts_layout(Wc, nslot, nt, G);
-  float* const edge = reinterpret_cast<float*>(smem + Ly.edge);  // [2][Wc + 2][last X, first X, first Y]
+  float* const edge = reinterpret_cast<float*>(smem + Ly.edge);  // [2][Wc + 2][last X, -, first X, first Y]
   double* t_x = reinterpret_cast<double*>(smem + Ly.tx);
   double* t_PL = reinterpret_cast<double*>(smem + Ly.tPL);
   double* t_tail = reinterpret_cast<double*>(smem + Ly.ttail);
@@ -215,7 +224,7 @@ __global__ void __launch_bounds__(32 * (kMaxChainWarps + kReduceWarps))
   const int Kmax = Kmax64 < (1LL << 30) ? (int)Kmax64 : 0;
   if (Kmax64 >= (1LL << 30) && tid == 0) set_status(p.status, kStatusKcap);
   for (int q = tid; q < (int)ts_hist(nslot); q += nthr) hist[q] = 0.0f;
-  for (int q = tid; q < 2 * 3 * (Wc + 2); q += nthr) edge[q] = 0.0f;
+  for (int q = tid; q < 2 * 4 * (Wc + 2); q += nthr) edge[q] = 0.0f;
   __syncthreads();  // the window tables and group pointers are read by every thread below
   // Group gq: its members (at most two) as float offsets of history rows,
   // its time, and a zero Kahan accumulator.  A member state s = m + M sigma
@@ -302,16 +311,16 @@ __global__ void __launch_bounds__(32 * (kMaxChainWarps + kReduceWarps))
       }
     }
   };
-  float* const eown = edge + 3 * (warp + 1);  // a chain warp's slot (parity 0)
-  const int epar = 3 * (Wc + 2);               // floats per parity
+  float* const eown = edge + 4 * (warp + 1);  // a chain warp's slot (parity 0)
+  const int epar = 4 * (Wc + 2);               // floats per parity
+  // One 8-byte store by the end lanes (lane 31: the last X, lane 0: the first
+  // X and Y), without a branch per lane.
+  const bool edge_lane = lane == 0 || lane == 31;
+  const int eoff = lane == 0 ? 2 : 0;
   auto write_edges = [&](int par, auto OC) {
     constexpr int O = decltype(OC)::value;
-    float* e = eown + par * epar;
-    if (lane == 31) e[0] = X[(QP - 1 + O) % P1].y;
-    if (lane == 0) {
-      e[1] = X[O % P1].x;
-      e[2] = Y[O % P1].x;
-    }
+    const float a = lane == 0 ? X[O % P1].x : X[(QP - 1 + O) % P1].y;
+    if (edge_lane) *reinterpret_cast<float2*>(eown + par * epar + eoff) = make_float2(a, Y[O % P1].x);
   };
   if (is_chain) {
     write_hist(2 * kHist - 1, std::integral_constant<int, 0>{});
@@ -326,14 +335,20 @@ __global__ void __launch_bounds__(32 * (kMaxChainWarps + kReduceWarps))
   // copy run the recurrence (one thread per time, chunks in jump order).
   int slo = 0, shi = -1;
   auto stage = [&](int ka, int kb, int ltid, int lnthr, int lwarp, int lW) {  // jumps [ka, kb], kb - ka < 32
+    const int ke = kb;
     kb = min(kb, Kmax);
     if (kb < ka) return;
     while (slo < nt && t_K[slo] < ka) ++slo;
     while (shi + 1 < nt && t_L[shi + 1] <= kb) ++shi;
     const int j = ka + lane;
-    for (int i = slo + lwarp; i <= shi; i += lW)
-      if (j <= kb && t_wb[i] && j >= t_L[i] && j <= t_K[i])
-        cp_async_elem(ring + i * kWStride + ((j - 1) & (kWRing - 1)), t_wb[i] + j);
+    // (0 outside a window, so that the readers need no test; ke: the chunk's
+    // last jump, beyond Kmax too.)
+    for (int i = slo + lwarp; i <= shi; i += lW) {
+      if (j > ke) continue;
+      float* const d = ring + i * kWStride + ((j - 1) & (kWRing - 1));
+      if (j < t_L[i] || j > t_K[i]) *d = 0.0f;
+      else if (t_wb[i]) cp_async_elem(d, t_wb[i] + j);
+    }
     cp_async_commit();
     for (int i = slo + ltid; i <= shi; i += lnthr) {
       if (!t_rec[i]) continue;
@@ -384,27 +399,17 @@ __global__ void __launch_bounds__(32 * (kMaxChainWarps + kReduceWarps))
     for (int gq = ga + rtid; gq < gb; gq += nred) {
       const int2 lq = gloc[gq];
       const int i = gtime[gq];
-      const int ta = max(k0, t_L[i]) - k0, tb = min(k1, t_K[i]) - k0;  // jumps of the window in the chunk
-      const unsigned live = ((2u << tb) - 1u) & ~((1u << ta) - 1u);
       const float4* wr = reinterpret_cast<const float4*>(ring + i * kWStride + wbase);
       const float4* ha = reinterpret_cast<const float4*>(hist + lq.x + hc);
       const float4* hb = reinterpret_cast<const float4*>(hist + lq.y + hc);
-      float s0 = 0.0f, s1 = 0.0f;
+      float2 s2 = make_float2(0.0f, 0.0f);  // even and odd jumps
 #pragma unroll
       for (int t4 = 0; t4 < kHist / 4; ++t4) {
         const float4 a = ha[t4], b = hb[t4], w = wr[t4];
-        const float va[4] = {a.x, a.y, a.z, a.w}, vb[4] = {b.x, b.y, b.z, b.w}, ww[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int t = 4 * t4 + u;
-          const float v = __fadd_rn(va[u], vb[u]);
-          if (live & (1u << t)) {
-            if (t & 1) s1 = __fmaf_rn(ww[u], v, s1);
-            else s0 = __fmaf_rn(ww[u], v, s0);
-          }
-        }
+        s2 = v_fma(make_float2(w.x, w.y), v_add(make_float2(a.x, a.y), make_float2(b.x, b.y)), s2);
+        s2 = v_fma(make_float2(w.z, w.w), v_add(make_float2(a.z, a.w), make_float2(b.z, b.w)), s2);
       }
-      const float s = __fadd_rn(s0, s1);
+      const float s = __fadd_rn(s2.x, s2.y);
       const float y = __fsub_rn(s, acc_c[gq]);
       const float a0 = acc_s[gq];
       const float tt = __fadd_rn(a0, y);
@@ -443,7 +448,9 @@ __global__ void __launch_bounds__(32 * (kMaxChainWarps + kReduceWarps))
       constexpr int ON = (O + P1 - 1) % P1;
       if (CHECK && k > Kmax) return;
       const float* e = eown + (t & 1) * epar;  // a warp's own slot is never read
-      const float eL = e[-3], eRX = e[4], eRY = e[5];
+      const float eL = e[-4];
+      const float2 eR = *reinterpret_cast<const float2*>(e + 6);
+      const float eRX = eR.x, eRY = eR.y;
       const float lastXy = X[(QP - 1 + O) % P1].y, lastXx = X[(QP - 1 + O) % P1].x;
       const float fXx = X[O % P1].x, fXy = X[O % P1].y, fYx = Y[O % P1].x, fYy = Y[O % P1].y;
       float lin = __shfl_up_sync(kFull, lastXy, 1);
@@ -489,9 +496,10 @@ __global__ void __launch_bounds__(32 * (kMaxChainWarps + kReduceWarps))
           rY[j] = v_fma(bY[j], Y[(j + ON) % P1], rY[j]);
         }
       }
-      write_hist(hc + t, std::integral_constant<int, ON>{});
       write_edges((t + 1) & 1, std::integral_constant<int, ON>{});
       chain_sync();
+      // (Behind the barrier: the reducers read the history after the hand-over.)
+      write_hist(hc + t, std::integral_constant<int, ON>{});
       ++k;
     };
     // Chunk q fills history half q mod 2 once the reducers have emptied it
