@@ -22,7 +22,7 @@
 // lanes of a warp did alike (roots and divisions, about 250 instructions per
 // window) runs a thread per window instead, and the FP64 reciprocals of 8
 // consecutive k are one reciprocal of their product and 8 multiplications.
-// Measured: 256 thetas x 50 times FP32 151 -> 108 us, 10^4 thetas x 5 times
+// Measured: 256 thetas x 50 times FP32 151 -> 89 us, 10^4 thetas x 5 times
 // FP64 756 -> 543 us, one theta x 5 times FP64 20 -> 12 us.
 //
 // Tolerance rule: a warp per window does everything (K is known only after the
@@ -519,7 +519,10 @@ __device__ double corner_rate(const PlanParams& p, int64_t M, int64_t N, int c, 
   return exit_rate(p.kind, M, p.P, m + M * q + M * rows * (c >> 2), th);
 }
 
-__global__ void __launch_bounds__(256) plan_kernel(PlanParams p) {
+// (80 registers at 256 threads, 3 CTAs an SM: at 116 registers and 2 CTAs, 10^4
+// thetas took 614 us instead of 550.)
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS, THREADS == 512 ? 2 : 3) plan_kernel(PlanParams p) {
   const int job = blockIdx.x;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   __shared__ double s_omega;
@@ -758,7 +761,14 @@ cudaError_t launch_plan(const PlanParams& p, cudaStream_t s) {
   if (p.B <= 0) return cudaSuccess;
   // A single instance by the paper's rule: a CTA per window.
   const int split = p.B == 1 && p.trunc_mode == MJP_TRUNC_PAPER ? (p.ntimes < 64 ? p.ntimes : 64) : 1;
-  plan_kernel<<<dim3((unsigned)p.B, (unsigned)split), 256, 0, s>>>(p);
+  // A warp per window and direction: above 8 windows, 8 warps take three and
+  // more turns at the scans.  Measured with 8 and 16 warps: 256 thetas x 50
+  // times 108 and 89 us, 152 thetas x 50 times (smaller x) 63 and 49 us; at 5 times 8 warps
+  // have one or two turns, and the third CTA per SM counts for more.
+  const int local = (p.ntimes + split - 1) / split;
+  const dim3 grid((unsigned)p.B, (unsigned)split);
+  if (local > 8) plan_kernel<512><<<grid, 512, 0, s>>>(p);
+  else plan_kernel<256><<<grid, 256, 0, s>>>(p);
   return cudaGetLastError();
 }
 
