@@ -527,6 +527,70 @@ __global__ void __launch_bounds__(kMaxT, 1) chain_reg1d_kernel(const ChainParams
     ++k;
   };
 
+  // A round that meets one window at most (always, for a single time): the
+  // window's sums stay in registers for the round, the same Kahan steps in the
+  // same order.  Summing in shared memory jump by jump cost ~1,850 cycles a
+  // jump (two dependent loads and two stores per pair, in order), this way
+  // ~450: 152 chains of 5,000 states and 20,000 jumps, FP32: 6.10 -> 5.13 ms,
+  // of 420 states: 3.04 -> 1.99 ms.
+  T2 as[QP];
+  float2 ac[QP];
+  int one_i = 0, one_L = 0, one_K = -1;
+  auto jump_one = [&](auto OC) {
+    constexpr int O = decltype(OC)::value, ON = (O + QP) % P1;
+    if (k > Kmax) return;
+    jump(OC);
+    if (k >= one_L && k <= one_K) {
+      const T w = ring[one_i * kStage1 + (k & (kStage1 - 1))];
+#pragma unroll
+      for (int j = 0; j < QP; ++j) {
+        const T2 v = r[(j + ON) % P1];
+        if constexpr (kComp) {
+          const float2 m1 = make_float2(-1.0f, -1.0f), w2 = make_float2(w, w);
+          const float2 y = __ffma2_rn(ac[j], m1, __fmul2_rn(w2, v));
+          const float2 t = __fadd2_rn(as[j], y);
+          ac[j] = __ffma2_rn(y, m1, __ffma2_rn(as[j], m1, t));
+          as[j] = t;
+        } else {
+          as[j] = v_make(f_fma(w, v.x, as[j].x), f_fma(w, v.y, as[j].y));
+        }
+      }
+    }
+    ++k;
+  };
+  auto round_one = [&](int i) {  // i < 0: no window is active
+    const int k0 = k;
+    one_i = max(i, 0);
+    one_L = i < 0 ? 0 : t_L[i];
+    one_K = i < 0 ? -1 : t_K[i];
+    const bool begun = one_L < k0 && one_K >= k0;
+#pragma unroll
+    for (int j = 0; j < QP; ++j) {
+      const int slot = (one_i * QP + j) * nthr + tid;
+      as[j] = begun ? acc_s[slot] : v_make((T)0, (T)0);
+      if (kComp) ac[j] = begun ? acc_c[slot] : make_float2(0.0f, 0.0f);
+    }
+    RotSeq<P1, 0, P1>::run(jump_one);
+    if (one_K < k0) return;
+    if (one_K >= k) {
+#pragma unroll
+      for (int j = 0; j < QP; ++j) {
+        const int slot = (one_i * QP + j) * nthr + tid;
+        acc_s[slot] = as[j];
+        if (kComp) acc_c[slot] = ac[j];
+      }
+      return;
+    }
+    T* const o = reinterpret_cast<T*>(p.out) + out_base + (int64_t)t_orig[one_i] * N + xb + xw;
+#pragma unroll
+    for (int j = 0; j < QP; ++j) {
+      T2 v = as[j];
+      if constexpr (kComp) v = v_make(__fsub_rn(as[j].x, ac[j].x), __fsub_rn(as[j].y, ac[j].y));
+      if ((omask >> (2 * j)) & 1u) o[y0 + j] = v.x;
+      if ((omask >> (2 * j + 1)) & 1u) o[y0 + QP + j] = v.y;
+    }
+  };
+
   // ---- the jump chain -------------------------------------------------------
   // Warps run rounds of P1 jumps without meeting: a warp window's halo (one
   // lane's run, R >= P1 states) goes stale from its outer edge at one state
@@ -574,7 +638,16 @@ __global__ void __launch_bounds__(kMaxT, 1) chain_reg1d_kernel(const ChainParams
   advance(kE, lo, hi);
   if (wact) accumulate(kE, lo, hi, std::integral_constant<int, 0>{});
   while (k <= Kmax) {
-    RotSeq<P1, 0, P1>::run(jump_acc);
+    while (lo < nt && t_K[lo] < k) ++lo;
+    int h1 = hi;
+    while (h1 + 1 < nt && t_L[h1 + 1] < k + P1) ++h1;
+    if (h1 <= lo) {
+      hi = h1;
+      if (wact) round_one(h1 == lo ? lo : -1);
+      else k = min(k + P1, Kmax + 1);
+    } else {
+      RotSeq<P1, 0, P1>::run(jump_acc);
+    }
     const int k_e = k - 1;
     if (k_e >= Kmax) break;
     defect();
