@@ -120,7 +120,7 @@ extern "C" {
                                    instance fits it (N_j <= 8 x 6,720 states FP32, 8 x 3,360 FP64), 1 = shared-memory
                                    kernel, 2 = register-resident kernel */
 #define MJP_OPT_HALO 8          /* batches, register-resident kernel: halo width h of an instance split over a cluster,
-                                   i.e. jumps between two halo exchanges (default 32; 1 .. 1024) */
+                                   i.e. jumps between two halo exchanges (default 64 FP32, 32 FP64; 1 .. 1024) */
 #define MJP_OPT_METHOD 9        /* expv_series method: 0 = R-MJP (Algorithm 2, default), 1 = fourth-order Runge-Kutta
                                    (Method #4), 2 = Krylov subspace steps (Method #5, Algorithm 3 with the full
                                    projection of Eq. Krylov_projection).  1 and 2: FP64 birth-death and two-state

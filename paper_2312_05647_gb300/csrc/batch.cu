@@ -66,7 +66,9 @@ struct mjp_batch {
   // register-resident kernel: 0 = automatic, 1 = shared-memory kernel only,
   // 2 = register kernel only (MJP_OPT_CHAIN)
   int chain = 0;
-  int reg_heavy_cluster = 4, reg_halo = 32;
+  int reg_heavy_cluster = 4;
+  int reg_halo = 0;   // halo of a cluster's CTAs (MJP_OPT_HALO), 0 = automatic
+  int halo_used = 0;  // what the groups were planned with
   double reg_heavy_factor = 1.0;
   int renorm = kDefectPeriod;  // FP32: exit-defect correction period (MJP_OPT_RENORM_PERIOD)
   int sms = 152;
@@ -154,8 +156,14 @@ int regroup_classic(mjp_batch* b) {
 // most kMaxRegCluster), heavy ones at least reg_heavy_cluster; one group per
 // cluster size, and six size classes of single-CTA instances (a CTA is as wide
 // as its group's largest instance needs, so classes keep idle threads few).
+// FP32 clusters carry a halo of 64 states: an exchange costs ~2,400 cycles
+// whatever the halo, 32 more states on each side 1 to 2% of the work.  Measured
+// with 32 and 64, means over five batches: 4,096 instances of up to 20,000
+// states 175.4 and 162.4 ms, 700 of them up to t = 3 23.9 and 22.1 ms.  FP64,
+// bound by its pipe, pays for every halo state and keeps 32.  (Clusters of 1, 2, 4 and 8 CTAs only: 20.6 ms for the 700,
+// but 181 ms for the 4,096; clusters launched before the single CTAs 181 ms.)
 // Returns MJP_ERR_UNSUPPORTED when some instance fits no cluster.
-int regroup_reg(mjp_batch* b) {
+int regroup_reg(mjp_batch* b, int halo) {
   double total = 0.0;
   for (double w : b->work) total += w;
   const double fair = total / std::max(1, b->sms);
@@ -164,11 +172,11 @@ int regroup_reg(mjp_batch* b) {
   Reg1dPlan rp;
   for (int j = 0; j < b->n; ++j) {
     int c = 1;
-    while (c <= kMaxRegCluster && !chain_reg1d_plan(b->precision, b->N[j], 1, c, b->reg_halo, &rp)) ++c;
+    while (c <= kMaxRegCluster && !chain_reg1d_plan(b->precision, b->N[j], 1, c, halo, &rp)) ++c;
     if (c > kMaxRegCluster) return fail(MJP_ERR_UNSUPPORTED, "an instance does not fit the register-resident chain");
     if (b->work[j] > b->reg_heavy_factor * fair)
       for (int ch = std::min(b->reg_heavy_cluster, kMaxRegCluster); ch > c; --ch)
-        if (chain_reg1d_plan(b->precision, b->N[j], 1, ch, b->reg_halo, &rp)) {
+        if (chain_reg1d_plan(b->precision, b->N[j], 1, ch, halo, &rp)) {
           c = ch;
           break;
         }
@@ -194,7 +202,7 @@ int regroup_reg(mjp_batch* b) {
     int64_t nmax = 0;
     for (int32_t j : g.jobs) nmax = std::max(nmax, b->N[j]);
     const int C = gi <= 5 ? 1 : gi - 4;
-    if (!chain_reg1d_plan(b->precision, nmax, 1, C, b->reg_halo, &g.rp))
+    if (!chain_reg1d_plan(b->precision, nmax, 1, C, halo, &g.rp))
       return fail(MJP_ERR_UNSUPPORTED, "a batch group does not fit the register-resident chain");
     g.cluster = C;
     g.threads = g.rp.threads;
@@ -211,7 +219,11 @@ int regroup_reg(mjp_batch* b) {
 
 int regroup(mjp_batch* b) {
   int rc = MJP_ERR_UNSUPPORTED;
-  if (b->chain != 1) rc = regroup_reg(b);
+  if (b->chain != 1) {
+    b->halo_used = b->reg_halo ? b->reg_halo : b->precision == MJP_FP64 ? 32 : 64;
+    rc = regroup_reg(b, b->halo_used);
+    if (rc && !b->reg_halo && b->halo_used > 32) rc = regroup_reg(b, b->halo_used = 32);
+  }
   if (rc && b->chain != 2) rc = regroup_classic(b);
   if (rc) return rc;
   b->grouped = true;
@@ -489,7 +501,7 @@ int expv_batch_tune(mjp_batch* b, void* out, void* stream, char* cfg, int cfg_le
       snprintf(cfg, (size_t)cfg_len,
                "{\"chain\": \"register\", \"heavy_cluster\": %d, \"heavy_factor\": %.2f, \"halo\": %d, "
                "\"ms\": %.4f, \"cluster_jobs\": %zu}",
-               b->reg_heavy_cluster, b->reg_heavy_factor, b->reg_halo, best, heavy);
+               b->reg_heavy_cluster, b->reg_heavy_factor, b->halo_used, best, heavy);
     else
       snprintf(cfg, (size_t)cfg_len,
                "{\"chain\": \"shared\", \"light_threads\": [%d, %d, %d], \"heavy_cluster\": %d, "
