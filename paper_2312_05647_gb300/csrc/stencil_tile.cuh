@@ -619,14 +619,17 @@ __global__ void __launch_bounds__(MAXT, 1) tile_kernel(const ChainParams p, cons
   // holds the jump.  A hand-over of the same parity reuses the slots and barriers: the
   // neighbour sends it only after it has received this CTA's pairs of the
   // hand-over in between, which left after the slots were read and the
-  // barriers armed again (a CTA barrier lies between).  After a wait that ran
-  // out (kStatusTimeout) the thread neither waits, arms nor sends any more.
+  // barriers armed again (a CTA barrier lies between).  When any thread's wait
+  // runs out (kStatusTimeout), the barrier that closes the hand-over tells the
+  // whole CTA (threads that send need not receive), and it neither sends, waits
+  // nor arms any more.  Its neighbours then run out at the next hand-over at
+  // the latest, which they have sent by then: every byte sent falls on a phase
+  // armed for it, and no more than these two phases can still be on their way.
   unsigned hpar = 0, hph = 0;  // parity of the hand-over; phase of each parity's barriers
-  bool hok = true;
-  unsigned hlost = 0;  // parity and phase of the wait that ran out
+  bool lost = false;           // the same in all threads of the CTA
   auto hand_send = [&]() {
     const unsigned slot0 = (unsigned)__cvta_generic_to_shared(hx) + hpar * 2u * hside;
-    if (owner && hok) {
+    if (owner && !lost) {
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         const int f = ty * R + r;
@@ -645,9 +648,15 @@ __global__ void __launch_bounds__(MAXT, 1) tile_kernel(const ChainParams p, cons
       }
     }
   };
+  // Ends with the CTA barrier after which the tile may be read.
   auto hand_recv = [&](int at) {
     T2* const tile = buf + at * bstride;
-    if ((rx_dn || rx_up) && hok) {
+    bool out = false;  // this thread's wait ran out
+    if (lost) {
+      __syncthreads();
+      return;
+    }
+    if (rx_dn || rx_up) {
       const unsigned ph = (hph >> hpar) & 1u;
       bool ok = !rx_dn || hbar_wait(hb + 8u * hpar, ph, p.wait_limit);
       if (ok && rx_up) ok = hbar_wait(hb + 16u + 8u * hpar, ph, p.wait_limit);
@@ -672,13 +681,13 @@ __global__ void __launch_bounds__(MAXT, 1) tile_kernel(const ChainParams p, cons
           tile[o0 + r * st] = S[r];
         }
       } else {
-        hok = false;
-        hlost = hpar | ph << 1;
+        out = true;
         set_status(p.status, kStatusTimeout);
       }
     }
     hph ^= 1u << hpar;
     hpar ^= 1u;
+    lost = __syncthreads_or(out) != 0;
   };
   int xleft = tg.period;
   if (LL) {
@@ -693,8 +702,9 @@ __global__ void __launch_bounds__(MAXT, 1) tile_kernel(const ChainParams p, cons
           hand_send();
           hand_recv(at);
           xleft = tg.period;
+        } else {
+          __syncthreads();
         }
-        __syncthreads();
       }
     };
     for (int kb = 0; kb <= Kmax; kb += JB) {
@@ -804,8 +814,9 @@ __global__ void __launch_bounds__(MAXT, 1) tile_kernel(const ChainParams p, cons
               break;
             }
             hand_recv(to);
+          } else {
+            __syncthreads();
           }
-          __syncthreads();
         }
       }
       // rho*_i += sum_j P_{kb+j} rho_{kb+j}, j = 1 .. J, for the windows that meet the block.
@@ -885,10 +896,7 @@ __global__ void __launch_bounds__(MAXT, 1) tile_kernel(const ChainParams p, cons
           }
         }
       }
-      if (sent) {
-        hand_recv(0);
-        __syncthreads();
-      }
+      if (sent) hand_recv(0);
       // The next chunk of weights, once no one reads the slots it takes (the
       // block's barriers lie behind the reads of the chunk before).
       if ((kb & (kc - 1)) == 0 && kb > 0 && kb + kc < Kmax) stage_chunk(kb + kc + 1);
@@ -896,14 +904,20 @@ __global__ void __launch_bounds__(MAXT, 1) tile_kernel(const ChainParams p, cons
   }
   cp_async_wait<0>();
   if (link) {
-    // No CTA leaves while a neighbour's pairs may be on their way to it: those
-    // of a wait that ran out may still come (bounded again).
-    if (!hok) {
-      constexpr long long kDrain = 1 << 16;
-      if (rx_dn) hbar_wait(hb + 8u * (hlost & 1u), hlost >> 1, kDrain);
-      if (rx_up) hbar_wait(hb + 16u + 8u * (hlost & 1u), hlost >> 1, kDrain);
-    }
+    // No CTA leaves while a neighbour's pairs may be on their way to it: after a
+    // wait that ran out, those of that hand-over and of the next one may still
+    // come.  Behind this barrier all of them have been sent; the waits (bounded
+    // again, 2 ms and more) end as soon as they have landed.
     cluster.sync();
+    if (lost) {
+      constexpr long long kDrain = 1 << 16;
+#pragma unroll 1
+      for (int q = 0; q < 2; ++q) {  // the next hand-over, then the one that ran out
+        const unsigned par = hpar ^ (unsigned)q, ph = ((hph >> par) & 1u) ^ (unsigned)q;
+        if (rx_dn) hbar_wait(hb + 8u * par, ph, kDrain);
+        if (rx_up) hbar_wait(hb + 16u + 8u * par, ph, kDrain);
+      }
+    }
   }
   if (!LL && any_rec && owner) {
     // Times whose K is above the cap (their weight is NaN) have no result.
