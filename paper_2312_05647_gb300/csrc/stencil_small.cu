@@ -15,8 +15,8 @@
 // reducers read jumps kb + 1 .. kb + 8, the chain writes kb + 9 .. kb + 16.
 //
 // Arithmetic per state is the sequence of stencil.cu; the sums are those of
-// stencil_tile.cuh (FP32: a chain of 8 multiply-adds, then a Kahan step; FP64:
-// one jump after the other).
+// stencil_tile.cuh (one jump after the other; FP32: a Kahan step for each
+// product).
 #include <algorithm>
 
 #include "chain_common.cuh"
@@ -225,12 +225,12 @@ __global__ void __launch_bounds__(1024, 1) chain_small_kernel(const ChainParams 
         const bool first = t_L[i] > kb, last = t_K[i] <= kb + kJ;
         if constexpr (kComp) {
           float2 a = first ? make_float2(0.0f, 0.0f) : acc32[(size_t)i * N + n];
-          float t = __fmul_rn(w[0], H[0]);
 #pragma unroll
-          for (int j = 1; j < kJ; ++j) t = __fmaf_rn(w[j], H[j], t);
-          const float y = __fsub_rn(t, a.y), s = __fadd_rn(a.x, y);
-          a.y = __fsub_rn(__fsub_rn(s, a.x), y);
-          a.x = s;
+          for (int j = 0; j < kJ; ++j) {
+            const float y = __fsub_rn(__fmul_rn(w[j], H[j]), a.y), s = __fadd_rn(a.x, y);
+            a.y = __fsub_rn(__fsub_rn(s, a.x), y);
+            a.x = s;
+          }
           if (last) finish(i, a.x, a.y);
           else acc32[(size_t)i * N + n] = a;
         } else {
@@ -280,11 +280,14 @@ cudaError_t launch_small(const ChainParams& p, const SmallPlan& sp, cudaStream_t
 // Up to 512 states (16 chain warps, as many reducers).  Two-state FP64 models
 // whose windows overlap so much that one SM's FP64 pipe is the bound (about
 // 1,200 cycles a jump) go to the tile kernel, which spreads them over a
-// cluster; birth-death models have no such alternative.  Measured, K about
-// 750, against the kernel that ran before (birth-death: stencil_reg1d.cu,
-// two-state: stencil_tile.cuh): N = 64 at 5 times FP64 626 -> 170 us, FP32
-// 389 -> 107; N = 512 at 5 times FP32 471 -> 157; two-state N_R = 33 at 5
-// times FP64 392 -> 220, N_R = 256 FP32 161 -> 161 (even).
+// cluster; birth-death models have no such alternative.  Measured with K =
+// 859 (us a call, planner included), birth-death against stencil_reg1d.cu: N =
+// 64 at 5 times FP64 676 -> 181, FP32 415 -> 119, at 20 times FP64 1,490 ->
+// 266, FP32 805 -> 142; N = 512 at 5 times FP64 1,121 -> 642, FP32 513 -> 184,
+// at 20 times FP64 2,629 -> 1,208, FP32 906 -> 285 (more overlapping windows
+// than the shared memory holds accumulators for go to stencil_reg1d.cu).
+// Two-state against stencil.cu: N_R = 64 at 5 times FP64 943 -> 258, FP32 852
+// -> 125, N_R = 256 FP32 961 -> 185 (against stencil_tile.cuh even there).
 bool chain_small_plan(int kind, int precision, int64_t M, int64_t N, int nt, double overlap, SmallPlan* out) {
   if (kind != MJP_BD1D && kind != MJP_TWOSTATE) return false;
   if (N > 512) return false;

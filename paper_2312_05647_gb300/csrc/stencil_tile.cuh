@@ -26,10 +26,11 @@
 // 24,000 cycles per jump.
 //
 // Transient distributions: the tile is J deep instead of double-buffered, so a
-// thread finds its values of the last J jumps there, and adds
-// sum_j P_{k+j} rho_{k+j} to an output once per J jumps (FP32: a fused
-// multiply-add chain, then one Kahan step; FP64: the same order of operations
-// as one jump at a time).  The accumulators of the windows that overlap stay
+// thread finds its values of the last J jumps there, and takes an output's
+// sum through J jumps at a time in registers (FP32: a Kahan step for each
+// product P_{k+j} rho_{k+j}; both precisions: the operations of one jump at a
+// time in their order.  A jump beyond the window's last one has weight 0; its
+// Kahan step leaves sum - compensation as it is).  The accumulators of the windows that overlap stay
 // in shared memory while they fit, the others in global memory.
 //
 // Clusters split row kinds by columns: the pairs at a boundary are pushed into
@@ -53,8 +54,9 @@
 // Measured against the shared-memory kernel (one GB300): autoregulatory
 // network 40 x 120, 152 thetas, 50 times, FP32 12.5 -> 2.0 ms; birth-death N =
 // 64, 10^4 thetas, FP64 7.61 -> 3.55 ms; two-state N_R = 131, one theta, FP64
-// 1.88 -> 1.03 ms; mRNA/protein 200 x 200, 20 times, FP32 463 -> 64 ms (15
-// CTAs instead of 4, 1,920 cycles per jump).
+// 1.88 -> 1.03 ms; mRNA/protein 200 x 200, 20 times, FP32 463 -> 66 ms (15
+// CTAs instead of 4, 0.95 us per jump; sums as multiply-add chains with one
+// Kahan step per J jumps took 63 ms, but are held in fewer bits).
 #pragma once
 
 #include <cooperative_groups.h>
@@ -876,10 +878,8 @@ __global__ void __launch_bounds__(MAXT, 1) tile_kernel(const ChainParams p, cons
             }
             constexpr int q = 0;
             if constexpr (kComp) {
-              float2 t = v_mul(v_make(w[0], w[0]), H[0][kPre ? r : q]);
 #pragma unroll
-              for (int j = 1; j < J; ++j) t = v_fma(v_make(w[j], w[j]), H[j][kPre ? r : q], t);
-              kahan_pair(t, s, c);
+              for (int j = 0; j < J; ++j) kahan_pair(v_mul(v_make(w[j], w[j]), H[j][kPre ? r : q]), s, c);
             } else {
 #pragma unroll
               for (int j = 0; j < J; ++j) s = v_fma(v_make(w[j], w[j]), H[j][kPre ? r : q], s);

@@ -35,7 +35,9 @@ const int* runs_of(int kind, int precision, bool ll, bool cl) {
 // of about 250 (row kinds) or 450 (grid kinds) cycles of latency and 15 per
 // pair and warp, 4 more per overlapping window (fitted on the 200 x 200
 // mRNA/protein box: 3 to 6 pairs per thread on 13 and 19 warps, 1,530 to 1,920
-// cycles without hand-overs, within 2%).  FP64: every operation holds a
+// cycles without hand-overs, within 2%; the fit dates from sums with one Kahan
+// step per J jumps, and 6 per window, nearer to a step per product, leaves all
+// but a few shapes as they are).  FP64: every operation holds a
 // scheduler's FP64 pipe for 64 cycles per warp.  A cluster barrier adds about
 // 1,000 cycles, a hand-over of halo rows about 1,200 (measured: 1,150 on 15
 // CTAs).
