@@ -7,8 +7,8 @@
 // padded stride, so that reading it is free of bank conflicts; the hidden
 // activations of the tile are broadcast from shared memory as float4.
 // Gradients have a kernel of their own (grad_kernel below), which writes one
-// partial per CTA; a second kernel sums the partials in a fixed order
-// (float-float) and applies Adam, so every result is run-to-run identical.  The
+// partial per CTA; a second kernel sums the partials in a fixed order (to
+// FP64's accuracy) and applies Adam, so every result is run-to-run identical.  The
 // network is tiny (17,281 parameters, 34 kflop per row forward): a step is
 // latency-bound, and FP32 FMA on the CUDA cores keeps the gradients exact
 // enough to check against FP64 backpropagation.
@@ -237,9 +237,9 @@ __global__ void __launch_bounds__(128) rows_kernel(const RowsParams p) {
 // Layer 2: two units of R / 4 rows per thread.  dL/dW2: one column of 64 rows
 // per thread; dL/dh1: one unit of R / 2 rows.  Bound: shared-memory reads
 // (about 8,000 wavefronts per CTA at R = 16) and latency.  Measured on 1,024
-// rows (64 CTAs): 22.8 -> 14.3 us against one thread per unit; the sums and
-// the Adam update 17.3 -> 5.6 us; 100 steps with the standardisation of 65,536
-// rows (342 -> ~15 us) 4.19 -> 1.77 ms.
+// rows (64 CTAs): 22.8 -> 14.3 us against one thread per unit; 100 steps with the
+// standardisation of 65,536 rows (342 -> ~15 us) and the sums below 4.19 -> 1.82
+// ms.
 template <int R>
 struct GradSmem {
   float W2[H * H];
@@ -464,28 +464,40 @@ struct AdamParams {
   double* loss;   // may be null
 };
 
-// Gradient = sum of the CTA partials in a fixed order, then Adam.  Four
-// threads share a parameter's partials (a quarter each) and add them in
-// float-float arithmetic (Knuth's TwoSum, error-free; the low parts' own
-// rounding is 2^-48 relative), then the quarters in order: the FP64 additions
-// of one thread per parameter held the FP64 pipe and a serial chain for 17 us
-// at 64 partials.  The last CTA sums the losses.
+// Gradient = sum of the CTA partials in a fixed order, then Adam.  Four threads
+// share a parameter's partials (a quarter each), then the quarters are added in
+// order.  Sums are kept as three FP32 numbers (a cascade of Knuth's TwoSum, which
+// is error-free: Ogita, Rump and Oishi's SumK with K = 3), ~72 bits, and rounded
+// once to FP64 and once to FP32, so they are no further from the exact sum than
+// one in FP64.  FP64 additions hold a pipe that is 64 times slower: 100 steps of
+// 1,024 rows took 2.17 ms with them, 1.71 ms this way (1.66 ms in two FP32
+// numbers).  TwoSum makes an infinity a NaN, so a sum that is not finite is
+// formed again in FP64.  The last CTA sums the losses.  The next step's gradient
+// may start only when the partials of this one are complete: started while they
+// were still being formed, its CTAs shared SMs with them or with each other
+// (100 steps of 2,048 rows 2.84 instead of 1.83 ms).
 constexpr int kAdamParts = 4, kAdamParams = 64;  // threads per parameter, parameters per CTA
-struct FloatFloat {
-  float hi, lo;
+struct Sum3 {
+  float hi, mid, lo;
 };
-__device__ __forceinline__ void ff_add_to(FloatFloat& a, float b, float blo) {
-  const float s = __fadd_rn(a.hi, b);
-  const float v = __fsub_rn(s, a.hi);
-  const float e = __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, v)), __fsub_rn(b, v));
-  a.hi = s;
-  a.lo = __fadd_rn(a.lo, __fadd_rn(e, blo));
+// a + b = s + e exactly.
+__device__ __forceinline__ float two_sum(float a, float b, float& e) {
+  const float s = __fadd_rn(a, b);
+  const float v = __fsub_rn(s, a);
+  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, v)), __fsub_rn(b, v));
+  return s;
+}
+__device__ __forceinline__ void add_to(Sum3& a, float b) {
+  float e, f;
+  a.hi = two_sum(a.hi, b, e);
+  a.mid = two_sum(a.mid, e, f);
+  a.lo = __fadd_rn(a.lo, f);
 }
 __global__ void __launch_bounds__(kAdamParts * kAdamParams) reduce_adam_kernel(const AdamParams q) {
-  __shared__ FloatFloat part[kAdamParts][kAdamParams];
+  __shared__ Sum3 part[kAdamParts - 1][kAdamParams];  // of all quarters but the first
   __shared__ double red[8];
-  cudaTriggerProgrammaticLaunchCompletion();
   cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
   if (blockIdx.x == gridDim.x - 1) {
     if (!q.loss) return;
     double l = 0.0;
@@ -497,7 +509,7 @@ __global__ void __launch_bounds__(kAdamParts * kAdamParams) reduce_adam_kernel(c
   const int k = threadIdx.x & (kAdamParams - 1), w = threadIdx.x / kAdamParams;
   const int p = blockIdx.x * kAdamParams + k;
   const int per = (q.nblk + kAdamParts - 1) / kAdamParts;
-  FloatFloat g{0.f, 0.f};
+  Sum3 g{0.f, 0.f, 0.f};
   if (p < NPAR) {
     const int b1 = min(q.nblk, (w + 1) * per);
     int b = w * per;
@@ -506,16 +518,25 @@ __global__ void __launch_bounds__(kAdamParts * kAdamParams) reduce_adam_kernel(c
 #pragma unroll
       for (int u = 0; u < 8; ++u) v[u] = q.partial[(size_t)(b + u) * NPAR + p];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) ff_add_to(g, v[u], 0.f);
+      for (int u = 0; u < 8; ++u) add_to(g, v[u]);
     }
-    for (; b < b1; ++b) ff_add_to(g, q.partial[(size_t)b * NPAR + p], 0.f);
+    for (; b < b1; ++b) add_to(g, q.partial[(size_t)b * NPAR + p]);
   }
-  part[w][k] = g;
+  if (w > 0) part[w - 1][k] = g;
   __syncthreads();
   if (w == 0 && p < NPAR) {
 #pragma unroll
-    for (int u = 1; u < kAdamParts; ++u) ff_add_to(g, part[u][k].hi, part[u][k].lo);
-    const float gf = __fadd_rn(g.hi, g.lo);
+    for (int u = 0; u < kAdamParts - 1; ++u) {
+      add_to(g, part[u][k].hi);
+      add_to(g, part[u][k].mid);
+      add_to(g, part[u][k].lo);
+    }
+    float gf = (float)((double)g.hi + ((double)g.mid + (double)g.lo));
+    if (!isfinite(gf)) {
+      double d = 0.0;
+      for (int b = 0; b < q.nblk; ++b) d += (double)q.partial[(size_t)b * NPAR + p];
+      gf = (float)d;
+    }
     if (q.grad) q.grad[p] = gf;
     if (q.apply) {
       const float m = q.b1 * q.m[p] + (1.f - q.b1) * gf;
@@ -562,15 +583,21 @@ cudaError_t launch_rows(const RowsParams& p, int64_t rows, cudaStream_t s) {
 
 int rows_per_cta(int64_t rows) { return rows <= 512 ? 8 : (rows <= 4096 ? 16 : 32); }
 
+// Up to half as many tiles as SMs ask for more than half of an SM's shared
+// memory, so that each has an SM to itself (100 steps of 512 rows, 64 tiles:
+// 1.65 -> 1.48 ms; of 1,536 rows, 96 tiles, 1.75 -> 1.83 ms).
 template <int R>
 cudaError_t launch_grad_rows(const RowsParams& p, int64_t rows, bool overlap, cudaStream_t s) {
+  constexpr size_t kAlone = 118 * 1024;
+  static_assert(sizeof(GradSmem<R>) <= kAlone, "a tile fits the larger request");
   static std::atomic<bool> ready{false};
   if (!ready.load()) {
-    const cudaError_t e = cudaFuncSetAttribute(grad_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GradSmem<R>));
+    const cudaError_t e = cudaFuncSetAttribute(grad_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kAlone);
     if (e != cudaSuccess) return e;
     ready.store(true);
   }
-  return launch_after(overlap, grad_kernel<R>, (int)((rows + R - 1) / R), 256, sizeof(GradSmem<R>), p, s);
+  const int64_t tiles = (rows + R - 1) / R;
+  return launch_after(overlap, grad_kernel<R>, (int)tiles, 256, tiles <= 152 / 2 ? kAlone : sizeof(GradSmem<R>), p, s);
 }
 
 cudaError_t launch_grad(const RowsParams& p, int64_t rows, bool overlap, cudaStream_t s) {

@@ -64,3 +64,16 @@ def test_training_repeats_to_the_bit(batch):
         losses = net.train(dp * 1.0, dy * 1.0, steps=40, batch=batch, seed=9, device_data=True)  # data just written
         runs.append((losses, net.get_params()[0]))
     assert np.array_equal(runs[0][0], runs[1][0]) and np.array_equal(runs[0][1], runs[1][1])
+
+
+@pytest.mark.parametrize("rows", [30, 700])
+def test_infinite_residual_gives_an_infinite_gradient(rows):
+    """The partials are summed as numbers are: one that overflowed makes the sum
+    of its sign infinite, not NaN (the output bias: dL/db3 = sum of dL/df)."""
+    from paper_2312_05647_gb300 import surrogate as S
+    psi, y = _data(rows)
+    y[rows // 2] = 1e39  # beyond FP32 when standardised
+    net = S.MLP(seed=0)
+    net.set_params(mlp.init_params(11).astype(np.float32), _vec({"mu_x": np.zeros(4), "sd_x": np.ones(4), "mu_y": 0.0, "sd_y": 1.0}))
+    loss, g = net.loss_grad(psi, y)
+    assert loss == np.inf and g[mlp.NPAR - 1] == -np.inf
