@@ -193,11 +193,12 @@ __device__ __forceinline__ FF ff_shfl_up(FF a, int d) {
 // the runs.  The unnormalised weights of [L, K] go to `put` when `store`;
 // returns (lane 0) the sum of all weights, that of k > K and, downward, w_L.
 //
-// FP32 chains: products and sums in float-float (relative error ~1e-14 over a
-// window of ~10^4 terms, far below the FP32 weights the chains read).
+// FP32 chains: products and a lane's sums in float-float (relative error ~1e-14
+// over a window of ~10^4 terms, far below the FP32 weights the chains read), the
+// lanes' sums added in FP64.
 constexpr int kRun = 8;
-struct FFSums {
-  FF all, tail, wL;
+struct Sums64 {
+  double all, tail, wL;
 };
 __device__ __forceinline__ FF ff_warp_incl_prod(FF v, int lane) {
 #pragma unroll
@@ -207,17 +208,11 @@ __device__ __forceinline__ FF ff_warp_incl_prod(FF v, int lane) {
   }
   return v;
 }
-__device__ __forceinline__ FF ff_warp_sum(FF v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1)
-    v = ff_add(v, FF{__shfl_xor_sync(kFull, v.hi, o), __shfl_xor_sync(kFull, v.lo, o)});
-  return v;
-}
 // I: 32-bit jump counts where they fit (a 64-bit integer's conversion to FP32
 // runs at the FP64 pipe's rate, one per weight).
 template <class I, class Put>
-__device__ FFSums dir_weights(int dir, FF xf, FF invx, I L, I K, I m, I R, int lane, bool store, Put& put) {
-  FFSums r{{0.0f, 0.0f}, {0.0f, 0.0f}, {1.0f, 0.0f}};
+__device__ Sums64 dir_weights(int dir, FF xf, FF invx, I L, I K, I m, I R, int lane, bool store, Put& put) {
+  FF all{0.0f, 0.0f}, tail{0.0f, 0.0f}, wL{1.0f, 0.0f};
   FF carry{1.0f, 0.0f};
   if (dir == 0) {
     for (I base = m + 1; base <= R; base += 32 * kRun) {
@@ -239,8 +234,8 @@ __device__ FFSums dir_weights(int dir, FF xf, FF invx, I L, I K, I m, I R, int l
         const I k = k0 + b;
         if (k <= R) {
           const FF w = ff_mul(pre, loc[b]);
-          r.all = ff_add(r.all, w);
-          if (k > K) r.tail = ff_add(r.tail, w);
+          all = ff_add(all, w);
+          if (k > K) tail = ff_add(tail, w);
           else if (store) put(k, w);
         }
       }
@@ -267,21 +262,23 @@ __device__ FFSums dir_weights(int dir, FF xf, FF invx, I L, I K, I m, I R, int l
         const I k = k0 - b;
         if (k >= L) {
           const FF w = ff_mul(pre, loc[b]);
-          r.all = ff_add(r.all, w);
+          all = ff_add(all, w);
           if (store) put(k, w);
           if (k == L) wl = w;
         }
       }
       if (base - L < 32 * kRun) {  // the run that holds L
         const int src = (int)((base - L) / kRun);
-        r.wL = FF{__shfl_sync(kFull, wl.hi, src), __shfl_sync(kFull, wl.lo, src)};
+        wL = FF{__shfl_sync(kFull, wl.hi, src), __shfl_sync(kFull, wl.lo, src)};
       }
       const FF last = ff_mul(pre, pr);
       carry = FF{__shfl_sync(kFull, last.hi, 31), __shfl_sync(kFull, last.lo, 31)};
     }
   }
-  r.all = ff_warp_sum(r.all);
-  if (dir == 0) r.tail = ff_warp_sum(r.tail);
+  Sums64 r;
+  r.all = warp_sum(ff_to(all));
+  r.tail = dir == 0 ? warp_sum(ff_to(tail)) : 0.0;
+  r.wL = ff_to(wL);
   return r;
 }
 
@@ -290,9 +287,6 @@ __device__ FFSums dir_weights(int dir, FF xf, FF invx, I L, I K, I m, I R, int l
 // stored copy) to FP64 precision.  Upward, x^b / (k0 (k0+1) ..) for the run's
 // positions b comes from one reciprocal of the product of all its k, multiplied
 // back from the run's end (products of 8 factors up to 2^40 stay finite).
-struct Sums64 {
-  double all, tail, wL;
-};
 template <class Put>
 __device__ Sums64 dir_weights64(int dir, double x, double invx, int64_t L, int64_t K, int64_t m, int64_t R, int lane,
                                 bool store, Put& put) {
@@ -565,12 +559,10 @@ __global__ void __launch_bounds__(THREADS, THREADS == 512 ? 2 : 3) plan_kernel(P
   __shared__ double s_x[kMaxTimes], s_invx[kMaxTimes];
   __shared__ long long s_L[kMaxTimes], s_K[kMaxTimes], s_R[kMaxTimes], s_off[kMaxTimes];
   __shared__ signed char s_kind[kMaxTimes];
-  // Sums of both directions, the tail and w_L (FP32 chains: as float-float in
-  // the same place), later 1 / W in s_sum[.][1]; x and 1 / x in float-float.
+  // Sums of both directions, the tail and w_L, later 1 / W in s_sum[.][1]; x and
+  // 1 / x in float-float (FP32 chains), later 1 / W and the tail.
   __shared__ double s_sum[kMaxTimes][2], s_tail[kMaxTimes], s_wL[kMaxTimes];
   __shared__ FF s_xf[kMaxTimes], s_invxf[kMaxTimes];
-  static_assert(sizeof(FF) == sizeof(double), "float-float sums share the doubles' place");
-  auto ff_at = [](double& d) -> FF& { return reinterpret_cast<FF&>(d); };
   __shared__ long long s_tot;
   static_assert(kMaxTimes <= 256, "a thread per window");
   const bool fp64 = p.fp64_weights || p.arena_fp64;
@@ -652,29 +644,25 @@ __global__ void __launch_bounds__(THREADS, THREADS == 512 ? 2 : 3) plan_kernel(P
     const int64_t L = s_L[i], K = s_K[i], m = (int64_t)floor(x), R = s_R[i];
     const long long off = abase + s_off[i] - L;
     const bool mode = dir == 0 && lane == 0 && place;  // the mode's own weight
+    Sums64 r;
     if (fp64) {
       auto put = [&](int64_t k, double w) {
         if (p.arena_fp64) reinterpret_cast<double*>(p.arena)[off + k] = w;
         else reinterpret_cast<float*>(p.arena)[off + k] = (float)w;
       };
       if (mode) put(m, 1.0);
-      const Sums64 r = dir_weights64(dir, x, s_invx[i], L, K, m, R, lane, place, put);
-      if (lane == 0) {
-        s_sum[i][dir] = r.all;
-        if (dir == 0) s_tail[i] = r.tail;
-        else s_wL[i] = r.wL;
-      }
+      r = dir_weights64(dir, x, s_invx[i], L, K, m, R, lane, place, put);
     } else {
       auto put = [&](int64_t k, FF w) { reinterpret_cast<float*>(p.arena)[off + k] = w.hi; };
       if (mode) put(m, FF{1.0f, 0.0f});
-      const FFSums r = R < (1LL << 30)
-                           ? dir_weights<int>(dir, s_xf[i], s_invxf[i], (int)L, (int)K, (int)m, (int)R, lane, place, put)
-                           : dir_weights<int64_t>(dir, s_xf[i], s_invxf[i], L, K, m, R, lane, place, put);
-      if (lane == 0) {
-        ff_at(s_sum[i][dir]) = r.all;
-        if (dir == 0) ff_at(s_tail[i]) = r.tail;
-        else ff_at(s_wL[i]) = r.wL;
-      }
+      r = R < (1LL << 30)
+              ? dir_weights<int>(dir, s_xf[i], s_invxf[i], (int)L, (int)K, (int)m, (int)R, lane, place, put)
+              : dir_weights<int64_t>(dir, s_xf[i], s_invxf[i], L, K, m, R, lane, place, put);
+    }
+    if (lane == 0) {
+      s_sum[i][dir] = r.all;
+      if (dir == 0) s_tail[i] = r.tail;
+      else s_wL[i] = r.wL;
     }
   }
   __syncthreads();
@@ -693,12 +681,6 @@ __global__ void __launch_bounds__(THREADS, THREADS == 512 ? 2 : 3) plan_kernel(P
       r.tail = 0.0;
       r.woff = -1;
       if (s_kind[tid] == 0) {
-        if (!fp64) {
-          s_sum[tid][0] = ff_to(ff_at(s_sum[tid][0]));
-          s_sum[tid][1] = ff_to(ff_at(s_sum[tid][1]));
-          s_tail[tid] = ff_to(ff_at(s_tail[tid]));
-          s_wL[tid] = ff_to(ff_at(s_wL[tid]));
-        }
         const double invW = __ddiv_rn(1.0, 1.0 + s_sum[tid][0] + s_sum[tid][1]);
         r.PL = __dmul_rn(s_wL[tid], invW);
         r.tail = __dmul_rn(s_tail[tid], invW);
