@@ -502,6 +502,17 @@ __device__ void plan_time(const PlanParams& p, double omega, double t, Win* dst,
   if (lane == 0) *dst = r;
 }
 
+// Poisson(L | x) of a window at x <= 250 in FP64, L x / i after another: the start
+// of the recurrence of an FP32 window without a stored copy, where w_L is too
+// small for float-float (w_L < 1e-30, for x between 70 and 220; its low part
+// falls below FP32's range, at x = 106 w_L itself, and every weight of the window
+// was off by as much as 1e-3).
+__device__ __noinline__ double poisson_start(double x, int64_t L) {
+  double P = exp(-x);
+  for (int64_t i = 1; i <= L; ++i) P = __dmul_rn(P, __ddiv_rn(x, (double)i));
+  return P;
+}
+
 // max_n e_n over the corners of the box: the last and last but one state of
 // every axis, both gene states (thread c < 8).
 __device__ double corner_rate(const PlanParams& p, int64_t M, int64_t N, int c, const double* th) {
@@ -682,7 +693,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == 512 ? 2 : 3) plan_kernel(P
       r.woff = -1;
       if (s_kind[tid] == 0) {
         const double invW = __ddiv_rn(1.0, 1.0 + s_sum[tid][0] + s_sum[tid][1]);
-        r.PL = __dmul_rn(s_wL[tid], invW);
+        r.PL = !fp64 && !place && s_wL[tid] < 1e-30 ? poisson_start(s_x[tid], s_L[tid]) : __dmul_rn(s_wL[tid], invW);
         r.tail = __dmul_rn(s_tail[tid], invW);
         if (place) r.woff = abase + s_off[tid];
         s_tail[tid] = r.tail;
