@@ -4,6 +4,8 @@
 
 #include <cuda_runtime.h>
 
+#include <atomic>
+#include <cstdint>
 #include <new>
 #include <stdexcept>
 #include <string>
@@ -52,6 +54,21 @@ inline int exception_status() noexcept {
       return ::mjp::fail(MJP_ERR_CUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); \
     }                                                                                    \
   } while (0)
+
+// Function attributes belong to a device: `set` runs once for each device that
+// is current at a call (`done`: a static of the caller, a bit per device; devices
+// beyond 64 every time), so that later launches, those of a graph capture among
+// them, issue none.  Threads that meet here set the same values twice.
+template <typename F>
+cudaError_t once_per_device(std::atomic<uint64_t>& done, F&& set) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const uint64_t bit = dev < 64 ? (uint64_t)1 << dev : 0;
+  if (done.load() & bit) return cudaSuccess;
+  if ((e = set()) == cudaSuccess) done.fetch_or(bit);
+  return e;
+}
 
 // Grow-only device buffer.  Growing synchronises the device first so that no
 // queued kernel still uses the old allocation.

@@ -590,12 +590,11 @@ template <int R>
 cudaError_t launch_grad_rows(const RowsParams& p, int64_t rows, bool overlap, cudaStream_t s) {
   constexpr size_t kAlone = 118 * 1024;
   static_assert(sizeof(GradSmem<R>) <= kAlone, "a tile fits the larger request");
-  static std::atomic<bool> ready{false};
-  if (!ready.load()) {
-    const cudaError_t e = cudaFuncSetAttribute(grad_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kAlone);
-    if (e != cudaSuccess) return e;
-    ready.store(true);
-  }
+  static std::atomic<uint64_t> done{0};
+  const cudaError_t e = once_per_device(done, [] {
+    return cudaFuncSetAttribute(grad_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kAlone);
+  });
+  if (e != cudaSuccess) return e;
   const int64_t tiles = (rows + R - 1) / R;
   return launch_after(overlap, grad_kernel<R>, (int)tiles, 256, tiles <= 152 / 2 ? kAlone : sizeof(GradSmem<R>), p, s);
 }

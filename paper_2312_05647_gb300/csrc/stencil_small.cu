@@ -20,6 +20,7 @@
 #include <algorithm>
 
 #include "chain_common.cuh"
+#include "host_util.h"
 #include "internal.cuh"
 
 namespace mjp {
@@ -264,13 +265,12 @@ __global__ void __launch_bounds__(1024, 1) chain_small_kernel(const ChainParams 
 
 template <typename T, int KIND>
 cudaError_t launch_small(const ChainParams& p, const SmallPlan& sp, cudaStream_t s) {
-  static int ready = 0;
+  static std::atomic<uint64_t> done{0};
   auto kern = chain_small_kernel<T, KIND>;
-  if (!ready) {
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    if (e != cudaSuccess) return e;
-    ready = 1;
-  }
+  const cudaError_t e = once_per_device(done, [&] {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+  });
+  if (e != cudaSuccess) return e;
   kern<<<1, sp.threads, sp.smem, s>>>(p, sp.nchain);
   return cudaGetLastError();
 }

@@ -66,6 +66,7 @@
 #include <type_traits>
 
 #include "chain_common.cuh"
+#include "host_util.h"
 #include "internal.cuh"
 #include "tile_plan.h"
 
@@ -991,15 +992,13 @@ __global__ void __launch_bounds__(MAXT, 1) tile_kernel(const ChainParams p, cons
 template <typename T, int KIND, bool LL, bool CL, int R, int GPT>
 cudaError_t tile_one(const ChainParams* p, const TilePlan& tp, cudaStream_t s) {
   auto kern = tile_kernel<T, KIND, LL, CL, R, GPT, tile_jumps(sizeof(T), R), tile_max_threads(sizeof(T), LL, CL, R)>;
-  // Attributes are set once per kernel, at their largest, so that launches
-  // during a graph capture issue none.
-  static std::atomic<bool> ready{false};
-  cudaError_t e;
-  if (!ready.load()) {
-    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTileSmemMax)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess) return e;
-    ready.store(true);
-  }
+  // Attributes are set at their largest.
+  static std::atomic<uint64_t> done{0};
+  cudaError_t e = once_per_device(done, [&] {
+    const cudaError_t m = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTileSmemMax);
+    return m != cudaSuccess ? m : cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  });
+  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)((p ? p->B : 1) * tp.cluster));
   cfg.blockDim = dim3((unsigned)tp.threads);
