@@ -66,6 +66,7 @@ struct mjp_model {
   int64_t nslices = 0;
   DevBuf d_slice_ptr, d_slice_len, d_col, d_val, d_diag, d_perm;
   DevBuf d_bar;                            // grid barrier of the one-launch CSR chain
+  bool csr_two = false;                    // the ring of vectors could not be allocated: two instead
   long long wait_limit = (long long)1 << 24;  // MJP_OPT_WAIT_LIMIT
   // workspace (scratch owned by the handle)
   DevBuf d_times, d_orig, d_win, d_info, d_theta, d_comp, d_status, d_ll;
@@ -244,30 +245,43 @@ int arena_prepare(mjp_model* m, const double* host_theta, int B, const double* t
 // The general-CSR chain: planner (which also forms the weight table), windows
 // back to the host (the number of launches is the largest K), rho0 into the
 // in-degree order, then one launch per jump and one per kCsrBlock jumps for the
-// outputs.  Leaves the outputs (times in ascending order, states in the
-// internal order) in m->d_outp.
+// outputs (a ring of nine vectors), or one launch per jump that also adds its
+// vector to the outputs (two vectors: MJP_OPT_CHAIN = 1, where nine take more
+// than 16 GiB, and where they cannot be allocated).  Leaves the outputs (times in
+// ascending order, states in the internal order) in m->d_outp.
 int csr_run(mjp_model* m, const void* rho0, const double* sorted_times, int nt, int trunc_mode, double tol,
             cudaStream_t s, std::vector<Win>* wins) {
   const size_t elt = m->precision == MJP_FP64 ? 8 : 4;
   const int64_t n = m->N;
-  // The ring of vectors: a block of jumps and the one being formed; two
-  // vectors where nine would take more than 16 GiB (and for the one-launch chain).
-  const int block = m->chain == 2 || (size_t)(kCsrBlock + 1) * elt * n > ((size_t)16 << 30) ? 1 : kCsrBlock;
-  const int nring = block + 1;
+  // The ring of vectors: a block of jumps and the one being formed.
+  constexpr int kRingVecs = kCsrBlock + 1;
+  bool two = m->chain != 0 || m->csr_two || (size_t)kRingVecs * elt * n > ((size_t)16 << 30);
   // Weights of a window: at most 20 sqrt(x) + 16 (x - 10 sqrt x .. x + 10 sqrt x + 10).
   double wcap = 2.0;
   // (Windows beyond the cap are refused below.)
   for (int i = 0; i < nt; ++i) wcap += 20.0 * std::sqrt(std::min(m->csr_omega * sorted_times[i], (double)m->kcap)) + 16.0;
   const int64_t wtab = (int64_t)wcap;
   int rc = 0;
-  if ((rc = ensure_status(m)) || (rc = m->d_times.ensure(sizeof(double) * nt)) ||
-      (rc = m->d_win.ensure(sizeof(Win) * nt)) || (rc = m->d_info.ensure(sizeof(JobInfo))) ||
-      (rc = m->d_rho2.ensure((size_t)nring * elt * n)) || (rc = m->d_outp.ensure(elt * (size_t)nt * n)) ||
-      (rc = m->d_woff.ensure(sizeof(int64_t) * nt)) || (rc = m->d_L.ensure(sizeof(int64_t) * nt)) ||
-      (rc = m->d_K.ensure(sizeof(int64_t) * nt)) || (rc = m->d_wtab.ensure(sizeof(double) * (size_t)(wtab + 2))) ||
-      (rc = m->d_arena_ctl.ensure(16)))
-    return rc;
-  if (m->precision == MJP_FP32 && (rc = m->d_comp.ensure(sizeof(float) * (size_t)nt * n))) return rc;
+  auto allocate = [&]() {
+    int rc = 0;
+    if ((rc = ensure_status(m)) || (rc = m->d_times.ensure(sizeof(double) * nt)) ||
+        (rc = m->d_win.ensure(sizeof(Win) * nt)) || (rc = m->d_info.ensure(sizeof(JobInfo))) ||
+        (rc = m->d_outp.ensure(elt * (size_t)nt * n)) ||
+        (rc = m->d_woff.ensure(sizeof(int64_t) * nt)) || (rc = m->d_L.ensure(sizeof(int64_t) * nt)) ||
+        (rc = m->d_K.ensure(sizeof(int64_t) * nt)) || (rc = m->d_wtab.ensure(sizeof(double) * (size_t)(wtab + 2))) ||
+        (rc = m->d_arena_ctl.ensure(16)) ||
+        (m->precision == MJP_FP32 && (rc = m->d_comp.ensure(sizeof(float) * (size_t)nt * n))))
+      return rc;
+    return m->d_rho2.ensure((size_t)(two ? 2 : kRingVecs) * elt * n);
+  };
+  rc = allocate();
+  if (rc == MJP_ERR_ALLOC && !two) {
+    cudaDeviceSynchronize();  // (a call before this one may still read the ring)
+    m->d_rho2.release();
+    two = m->csr_two = true;
+    rc = allocate();
+  }
+  if (rc) return rc;
   MJP_CUDA(cudaMemcpyAsync(m->d_times.p, sorted_times, sizeof(double) * nt, cudaMemcpyHostToDevice, s));
   MJP_CUDA(cudaMemsetAsync(m->d_arena_ctl.p, 0, 16, s));
   PlanParams pp = {};
@@ -333,25 +347,46 @@ int csr_run(mjp_model* m, const void* rho0, const double* sorted_times, int nt, 
     cp.wait_limit = m->wait_limit;
     cp.status = m->d_status.as<int>();
     MJP_CUDA(launch_csr_chain(m->precision, cp, s));
+  } else if (two) {
+    CsrJumpParams jp = {};
+    jp.n = n; jp.nslices = m->nslices;
+    jp.slice_ptr = m->d_slice_ptr.as<int64_t>(); jp.slice_len = m->d_slice_len.as<int32_t>();
+    jp.col = m->d_col.as<int32_t>(); jp.val = m->d_val.p; jp.diag = m->d_diag.p;
+    jp.wtab = m->d_wtab.as<double>(); jp.woff = m->d_woff.as<int64_t>();
+    jp.L = m->d_L.as<int64_t>(); jp.K = m->d_K.as<int64_t>();
+    jp.out = m->d_outp.p; jp.comp = m->d_comp.as<float>();
+    int lo = 0, hi = -1;  // times whose window holds jump k - 1 (ascending times)
+    for (int64_t k = 1; k <= kmax + 1; ++k) {
+      const int64_t kp = k - 1;
+      while (lo < nt && K[lo] < kp) ++lo;
+      while (hi + 1 < nt && L[hi + 1] <= kp) ++hi;
+      jp.k = k;
+      jp.jump = k <= kmax;
+      jp.tlo = lo;
+      jp.thi = hi;
+      jp.rho_prev = rho + ((kp & 1) ? elt * n : 0);
+      jp.rho_next = rho + ((kp & 1) ? 0 : elt * n);
+      MJP_CUDA(launch_csr_jump(m->precision, jp, s));
+    }
   } else {
     CsrStepParams jp = {};
     jp.n = n;
     jp.slice_ptr = m->d_slice_ptr.as<int64_t>(); jp.slice_len = m->d_slice_len.as<int32_t>();
     jp.col = m->d_col.as<int32_t>(); jp.val = m->d_val.p; jp.diag = m->d_diag.p;
     CsrSumParams sp = {};
-    sp.n = n; sp.nring = nring; sp.ring = rho;
+    sp.n = n; sp.nring = kRingVecs; sp.ring = rho;
     sp.wtab = m->d_wtab.as<double>(); sp.woff = m->d_woff.as<int64_t>();
     sp.L = m->d_L.as<int64_t>(); sp.K = m->d_K.as<int64_t>();
     sp.out = m->d_outp.p; sp.comp = m->d_comp.as<float>();
     int lo = 0, hi = -1;  // times whose window meets the block (ascending times)
     for (int64_t k = 0; k <= kmax; ++k) {
       if (k > 0) {
-        jp.rho_prev = rho + (size_t)((k - 1) % nring) * elt * n;
-        jp.rho_next = rho + (size_t)(k % nring) * elt * n;
+        jp.rho_prev = rho + (size_t)((k - 1) % kRingVecs) * elt * n;
+        jp.rho_next = rho + (size_t)(k % kRingVecs) * elt * n;
         MJP_CUDA(launch_csr_step(m->precision, jp, s));
       }
-      if ((k + 1) % block != 0 && k != kmax) continue;
-      sp.k0 = k / block * block;
+      if ((k + 1) % kCsrBlock != 0 && k != kmax) continue;
+      sp.k0 = k / kCsrBlock * kCsrBlock;
       sp.count = (int)(k - sp.k0 + 1);
       while (lo < nt && K[lo] < sp.k0) ++lo;
       while (hi + 1 < nt && L[hi + 1] <= k) ++hi;

@@ -22,6 +22,10 @@
 // step per jump), instead of every jump reading and writing every active
 // output.
 //
+// Where only two vectors are held (MJP_OPT_CHAIN = 1, more than 16 GiB for nine, or
+// no memory for them), the launch of a jump adds the vector it reads to the active
+// outputs.
+//
 // Alternative (MJP_OPT_CHAIN = 2): the whole chain in one cooperative launch
 // (all CTAs co-resident), the outputs accumulated at every jump, jumps
 // separated by a software grid barrier whose waits are bounded (a CTA that
@@ -134,6 +138,11 @@ __device__ __forceinline__ void csr_jump_body(const CsrJumpParams& p) {
       nxt[r] = y;
     }
   }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(512) csr_jump_kernel(CsrJumpParams p) {
+  csr_jump_body<T>(p);
 }
 
 // One jump, a thread per state: its first kCsrPre entries are in registers
@@ -375,6 +384,14 @@ cudaError_t launch_csr_sum(int precision, const CsrSumParams& p, cudaStream_t s)
   const int64_t grid = (p.n + 255) / 256;
   return precision == MJP_FP64 ? launch_dependent(csr_sum_kernel<double>, grid, p, s)
                                : launch_dependent(csr_sum_kernel<float>, grid, p, s);
+}
+
+cudaError_t launch_csr_jump(int precision, const CsrJumpParams& p, cudaStream_t s) {
+  const int block = 512;
+  const int grid = grid_for(p.nslices * 32, block);
+  if (precision == MJP_FP64) csr_jump_kernel<double><<<grid, block, 0, s>>>(p);
+  else csr_jump_kernel<float><<<grid, block, 0, s>>>(p);
+  return cudaGetLastError();
 }
 
 template <typename T>

@@ -149,7 +149,7 @@ struct CsrSumParams {
   float* comp;               // FP32 Kahan compensation, ntimes x n
 };
 
-// One jump of the general-CSR chain in one launch (csr.cu).
+// One jump of the general-CSR chain and the sums of the vector it reads (csr.cu).
 struct CsrJumpParams {
   int64_t n, nslices;
   const int64_t* slice_ptr;  // first entry of each slice
@@ -171,7 +171,7 @@ struct CsrJumpParams {
 };
 
 // The whole general-CSR chain in one cooperative launch (csr.cu): every jump
-// of csr_jump_kernel's body, then a grid-wide barrier with a bounded wait.
+// of csr_jump_body, then a grid-wide barrier with a bounded wait.
 struct CsrChainParams {
   CsrJumpParams j;           // k, jump, tlo, thi, rho_prev and rho_next are set per jump in the kernel
   int ntimes;
@@ -309,6 +309,7 @@ cudaError_t launch_permute_out(int precision, const void* src, const int32_t* pe
                                int ntimes, const int32_t* orig, cudaStream_t s);
 cudaError_t launch_csr_step(int precision, const CsrStepParams& p, cudaStream_t s);
 cudaError_t launch_csr_sum(int precision, const CsrSumParams& p, cudaStream_t s);
+cudaError_t launch_csr_jump(int precision, const CsrJumpParams& p, cudaStream_t s);
 cudaError_t launch_csr_chain(int precision, const CsrChainParams& p, cudaStream_t s);
 cudaError_t launch_csr_loglik(const void* outp, int precision, int64_t n, const int64_t* gptr, int ntimes,
                               const double* counts, const int64_t* mptr, const int32_t* members,

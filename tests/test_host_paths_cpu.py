@@ -92,3 +92,36 @@ def test_transient_distributions_on_a_second_device(L, kind, dims, theta, nt, pr
         h = _stencil(L, kind, dims, theta, prec)
         _ok(L, _series(L, h, n, np.linspace(0.1, 5.0, nt), prec))
         L.rate_model_destroy(h)
+
+
+def _csr(L, n, prec):
+    """A ring of n states."""
+    h = ctypes.c_void_p()
+    rp, col, rate = np.arange(n + 1, dtype=np.int64), ((np.arange(n) + 1) % n).astype(np.int32), np.ones(n)
+    _ok(L, L.rate_model_create_csr(ctypes.byref(h), n, _p(rp, capi._i64p), _p(col, capi._i32p), _p(rate, capi._f64p), prec))
+    return h
+
+
+@pytest.mark.parametrize("prec", [1, 2])
+def test_general_matrix_runs_on_two_vectors_where_nine_do_not_fit(L, prec):
+    n, elt = 200000, 4 if prec == 1 else 8
+    out = (2 * elt if prec == 1 else elt) * n  # one output and, in FP32, its compensation
+    for spare, rc in ((9 * elt * n, 0), (3 * elt * n, 0), (elt * n, -3)):
+        L.fake_memory(1 << 40)
+        h = _csr(L, n, prec)
+        L.fake_memory(out + spare + (1 << 16))
+        assert _series(L, h, n, [0.5], prec) == rc
+        if rc == 0:
+            before = L.fake_mallocs()
+            _ok(L, _series(L, h, n, [0.5], prec))
+            assert L.fake_mallocs() == before  # nothing is tried again
+        L.rate_model_destroy(h)
+
+
+def test_general_matrix_gives_up_its_ring_for_more_outputs(L):
+    n = 200000
+    h = _csr(L, n, 2)
+    L.fake_memory(8 * n * 10 + (1 << 16))
+    _ok(L, _series(L, h, n, [0.5], 2))
+    _ok(L, _series(L, h, n, [0.5, 1.0, 1.5, 2.0], 2))  # 4 + 9 vectors do not fit, 4 + 2 do
+    L.rate_model_destroy(h)
