@@ -10,7 +10,8 @@
 // so every index and value load is one coalesced 128/256-byte transaction and
 // the sorting keeps padding negligible.  The diagonal 1 - e_n/Omega is a
 // separate array.  rho (4 MB for 2^20 FP32 states) stays resident in L2;
-// neighbour values are gathered with read-only loads.
+// neighbour values are gathered with ordinary loads (in the one-launch chain other
+// CTAs of the same launch write them, which read-only loads do not allow).
 //
 // Default: one launch per jump (rho_k = rho_{k-1} B, Algorithm 2's loop body;
 // rho_{k+1} depends on all of rho_k, so jumps are separated grid-wide).  Each
@@ -72,8 +73,8 @@ __device__ __forceinline__ void csr_jump_body(const CsrJumpParams& p) {
   const int lane = threadIdx.x & 31;
   const int64_t gwarp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const T* __restrict__ cur = reinterpret_cast<const T*>(p.rho_prev);
-  T* __restrict__ nxt = reinterpret_cast<T*>(p.rho_next);
+  const T* cur = reinterpret_cast<const T*>(p.rho_prev);  // (no read-only loads: see above)
+  T* nxt = reinterpret_cast<T*>(p.rho_next);
   const T* __restrict__ val = reinterpret_cast<const T*>(p.val);
   const T* __restrict__ diag = reinterpret_cast<const T*>(p.diag);
   T* __restrict__ out = reinterpret_cast<T*>(p.out);
@@ -124,7 +125,7 @@ __device__ __forceinline__ void csr_jump_body(const CsrJumpParams& p) {
         const int32_t c0 = __ldg(p.col + e), c1 = __ldg(p.col + e + 32), c2 = __ldg(p.col + e + 64),
                       c3 = __ldg(p.col + e + 96);
         const T a0 = __ldg(val + e), a1 = __ldg(val + e + 32), a2 = __ldg(val + e + 64), a3 = __ldg(val + e + 96);
-        const T g0 = __ldg(cur + c0), g1 = __ldg(cur + c1), g2 = __ldg(cur + c2), g3 = __ldg(cur + c3);
+        const T g0 = cur[c0], g1 = cur[c1], g2 = cur[c2], g3 = cur[c3];
         y = fma_t(a0, g0, y);
         y = fma_t(a1, g1, y);
         y = fma_t(a2, g2, y);
@@ -133,7 +134,7 @@ __device__ __forceinline__ void csr_jump_body(const CsrJumpParams& p) {
       for (; j < width; ++j) {
         const int64_t e = base + (int64_t)j * 32;
         const int32_t c = __ldg(p.col + e);
-        y = fma_t(__ldg(val + e), __ldg(cur + c), y);
+        y = fma_t(__ldg(val + e), cur[c], y);
       }
       nxt[r] = y;
     }
