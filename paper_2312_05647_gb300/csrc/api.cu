@@ -246,16 +246,16 @@ int arena_prepare(mjp_model* m, const double* host_theta, int B, const double* t
 // back to the host (the number of launches is the largest K), rho0 into the
 // in-degree order, then one launch per jump and one per kCsrBlock jumps for the
 // outputs (a ring of nine vectors), or one launch per jump that also adds its
-// vector to the outputs (two vectors: MJP_OPT_CHAIN = 1, where nine take more
-// than 16 GiB, and where they cannot be allocated).  Leaves the outputs (times in
-// ascending order, states in the internal order) in m->d_outp.
+// vector to the outputs (two vectors: where nine take more than 16 GiB, and where
+// they cannot be allocated; 2^20 states FP32 34.7 instead of 32.6 ms).  Leaves the
+// outputs (times in ascending order, states in the internal order) in m->d_outp.
 int csr_run(mjp_model* m, const void* rho0, const double* sorted_times, int nt, int trunc_mode, double tol,
             cudaStream_t s, std::vector<Win>* wins) {
   const size_t elt = m->precision == MJP_FP64 ? 8 : 4;
   const int64_t n = m->N;
   // The ring of vectors: a block of jumps and the one being formed.
   constexpr int kRingVecs = kCsrBlock + 1;
-  bool two = m->chain != 0 || m->csr_two || (size_t)kRingVecs * elt * n > ((size_t)16 << 30);
+  bool two = m->chain == 2 || m->csr_two || (size_t)kRingVecs * elt * n > ((size_t)16 << 30);
   // Weights of a window: at most 20 sqrt(x) + 16 (x - 10 sqrt x .. x + 10 sqrt x + 10).
   double wcap = 2.0;
   // (Windows beyond the cap are refused below.)
@@ -1209,10 +1209,13 @@ int loglik(mjp_model* m, const mjp_obs* obs, const double* theta, int B, double*
 
 }  // extern "C"
 
-// ---- internal accessors for the sampler (not part of the C ABI) -----------
+// ---- internal accessors for the sampler and tests (not part of the C ABI) -----------
 namespace mjp {
 
 int model_kind(const mjp_model* m) { return m->kind; }
+
+// As if the ring of vectors of a general rate matrix could not be allocated.
+void model_csr_two(mjp_model* m) { m->csr_two = true; }
 
 // Wait for `s`, grow the weight arena if a window overflowed it, then return
 // and clear the device status word (MJP_OK when nothing was flagged).  A
