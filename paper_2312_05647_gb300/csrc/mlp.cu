@@ -27,7 +27,7 @@ using namespace mjp::mlp;
 
 struct mjp_mlp {
   DevBuf P, m, v, norm;
-  DevBuf normp;  // column sums of the standardisation
+  DevBuf normp;  // column sums of the standardisation (allocated with the network: fitting takes no memory)
   DevBuf partial, loss_part, psi, y, out, losses, grad, scalar;
   int64_t t = 0;
 };
@@ -615,8 +615,6 @@ int launch_fit_norm(mjp_mlp* net, const double* psi, const double* y, int64_t n,
     MJP_CUDA(cudaGetLastError());
     return MJP_OK;
   }
-  int rc = net->normp.ensure(sizeof(double) * 2 * 5 * kNormCtas);
-  if (rc) return rc;
   double* sums = net->normp.as<double>();
   double* squares = sums + 5 * kNormCtas;
   norm_part_kernel<<<kNormCtas, 256, 0, s>>>(psi, y, n, 0, nullptr, sums);
@@ -672,7 +670,8 @@ int mjp_mlp_create(mjp_mlp** out, uint64_t seed) try {
   mjp_mlp* net = new mjp_mlp();
   int rc;
   if ((rc = net->P.ensure(sizeof(float) * NPAR)) || (rc = net->m.ensure(sizeof(float) * NPAR)) ||
-      (rc = net->v.ensure(sizeof(float) * NPAR)) || (rc = net->norm.ensure(sizeof(Norm)))) {
+      (rc = net->v.ensure(sizeof(float) * NPAR)) || (rc = net->norm.ensure(sizeof(Norm))) ||
+      (rc = net->normp.ensure(sizeof(double) * 2 * 5 * kNormCtas))) {
     mjp_mlp_destroy(net);
     return rc;
   }

@@ -125,3 +125,15 @@ def test_general_matrix_gives_up_its_ring_for_more_outputs(L):
     _ok(L, _series(L, h, n, [0.5], 2))
     _ok(L, _series(L, h, n, [0.5, 1.0, 1.5, 2.0], 2))  # 4 + 9 vectors do not fit, 4 + 2 do
     L.rate_model_destroy(h)
+
+
+def test_standardisation_of_device_data_takes_no_memory(L):
+    """So that it can be captured in a graph on a new network."""
+    n = 9000
+    psi, y = np.zeros((n + 1, 4)), np.zeros(n)
+    net = _net(L)
+    base = psi.ctypes.data + (-psi.ctypes.data) % 16
+    before = L.fake_mallocs()
+    _ok(L, L.mjp_mlp_fit_norm(net, base, y.ctypes.data, n, capi.PTR_DEVICE, None))
+    assert L.fake_mallocs() == before
+    L.mjp_mlp_destroy(net)

@@ -77,3 +77,21 @@ def test_infinite_residual_gives_an_infinite_gradient(rows):
     net.set_params(mlp.init_params(11).astype(np.float32), _vec({"mu_x": np.zeros(4), "sd_x": np.ones(4), "mu_y": 0.0, "sd_y": 1.0}))
     loss, g = net.loss_grad(psi, y)
     assert loss == np.inf and g[mlp.NPAR - 1] == -np.inf
+
+
+def test_standardisation_is_captured_on_a_new_network():
+    import ctypes
+    import torch
+    from paper_2312_05647_gb300 import capi
+    from paper_2312_05647_gb300 import surrogate as S
+    psi, y = _data(5000)
+    dp, dy = torch.tensor(psi, device="cuda"), torch.tensor(y, device="cuda")
+    net = S.MLP(seed=1)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        capi.check(capi.lib().mjp_mlp_fit_norm(net._h, ctypes.c_void_p(dp.data_ptr()), ctypes.c_void_p(dy.data_ptr()), 5000,
+                                               capi.PTR_DEVICE, ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)))
+    g.replay()
+    torch.cuda.synchronize()
+    np.testing.assert_allclose(net.get_params()[1], _vec(mlp.fit_norm(psi, y)), rtol=1e-12, atol=1e-15)
