@@ -1,0 +1,56 @@
+"""FP64 log-likelihoods of many thetas: the automatic chain against the
+shared-memory chain (MJP_OPT_CHAIN = 1) on both sides of the rule that chooses
+between them (csrc/tile_plan.cu, tile_pays64), in value and in time."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+TS, MP, AR = 2, 3, 5
+TH = {TS: [9.0, 0.7, 2.0, 1.0], MP: [3.0, 0.5, 1.5, 0.2], AR: [4.0, 0.5, 0.6, 0.1, 0.4, 0.05]}
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import torch
+    from paper_2312_05647_gb300 import build as lib_build
+    lib_build.build()
+    torch.cuda.set_device(0)
+
+
+def _ms(f):
+    import torch
+    f()
+    best = np.inf
+    for _ in range(4):
+        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        torch.cuda.synchronize()
+        a.record()
+        f()
+        b.record()
+        torch.cuda.synchronize()
+        best = min(best, a.elapsed_time(b))
+    return best
+
+
+@pytest.mark.parametrize("kind,dims,B,nt,per", [(MP, [120, 90], 152, 13, 100), (MP, [120, 90], 16, 13, 100), (MP, [64, 64], 152, 5, 20),
+                                                (MP, [231, 26], 417, 12, 43), (TS, [131], 1000, 5, 20), (TS, [70], 7128, 8, 9),
+                                                (AR, [110, 50], 2017, 5, 4), (AR, [40, 61], 152, 13, 50)])
+def test_automatic_chain_agrees_and_is_not_slower(kind, dims, B, nt, per):
+    import torch
+    import paper_2312_05647_gb300 as mjp
+    n = int(np.prod(dims)) * (2 if kind in (TS, AR) else 1)
+    gen = np.random.default_rng(B)
+    ob = [([np.sort(gen.choice(n, 2, replace=False)) for _ in range(per)], np.ones(per)) for _ in range(nt)]
+    obs = mjp.Obs(n, np.linspace(0.05, 0.5, nt), ob, np.full(n, 1.0 / n))
+    th = torch.tensor(np.asarray(TH[kind]) * gen.uniform(0.95, 1.05, (B, len(TH[kind]))), device="cuda")
+    ll, ms = {}, {}
+    for chain in (0, 1):
+        m = mjp.Model(kind, dims, TH[kind], 2)
+        m.set_option(mjp.OPT_CHAIN, chain)
+        ll[chain] = mjp.loglik(m, obs, th).cpu().numpy()
+        m.check()
+        ms[chain] = _ms(lambda: mjp.loglik(m, obs, th))
+    assert np.isfinite(ll[1]).all()
+    assert np.all(np.abs(ll[0] - ll[1]) <= nt * per * 1e-14 + 1e-12)
+    # The estimates are within 25%; the cases of the old choice were 1.25 to 2 times slower.
+    assert ms[0] <= 1.15 * ms[1], ms
