@@ -1149,10 +1149,9 @@ int loglik(mjp_model* m, const mjp_obs* obs, const double* theta, int B, double*
   bool use_tile = !use_reg && !use_ts && m->chain == 0 && m->cluster == 0 && m->threads == 0 &&
                   m->kcap <= (1 << 30) - 1 &&
                   tile_plan(m->kind, m->precision, true, m->M, m->P, nt, obs->G, obs->maxmem, B, overlap, &xp);
-  if (use_tile && m->precision == MJP_FP64 && m->kind != MJP_BD1D && B > 1 &&
-      stencil_config(m, 1, nt, obs->G, nmem_list, &C, &T, &slab) == MJP_OK)
-    use_tile = tile_pays64(m->kind, m->M, xp, nt, obs->G, B, overlap, C, T, slab,
-                           chain_stencil_smem(m->kind, m->precision, 1, m->M, m->P, slab, nt, obs->G, nmem_list));
+  if (use_tile && B > 1 && stencil_config(m, 1, nt, obs->G, nmem_list, &C, &T, &slab) == MJP_OK)
+    use_tile = tile_pays(m->kind, m->precision, m->M, xp, nt, obs->G, B, overlap, C, T, slab,
+                         chain_stencil_smem(m->kind, m->precision, 1, m->M, m->P, slab, nt, obs->G, nmem_list));
   if (!use_reg && !use_ts && !use_tile && (rc = stencil_config(m, 1, nt, obs->G, nmem_list, &C, &T, &slab))) return rc;
   if ((rc = ensure_status(m))) return rc;
   if ((rc = m->d_win.ensure(sizeof(Win) * (size_t)nt * B))) return rc;

@@ -141,70 +141,83 @@ bool tile_plan(int kind, int precision, bool ll, int64_t M, int64_t P, int nt, i
   return best_shape(kind, precision, ll, M, P, nt, G, maxmem, B, overlap, 8, out);
 }
 
-// FP64 log-likelihoods of more CTAs than SMs are bound by the FP64 pipe, and there
-// the tile kernel's halo pair rows (half of its work where a CTA holds four), its
-// cluster barriers and its 96 to 160 registers a thread can cost more than it
-// saves against stencil.cu, which holds 2 to 16 times the states per CTA in 64
-// registers.  Both sides are estimated: an SM serves its CTAs in batches of as many
-// as it holds, a batch takes the latency of a jump or the work of its CTAs.
-// Constants fitted to 4,000 calls (two-state models of 2 to 950 columns,
-// mRNA/protein boxes of up to 300 x 300, autoregulatory ones of up to 120 x 200, 1 to 8,000 thetas, 1 to 100 times, up to
-// 6,000 groups); 80% of the estimates are within 25%.  Of those calls 15.6% of the
-// mRNA/protein ones on clusters took longer than stencil.cu (at worst 2.1 times),
-// with this rule 2% (1.29 times); two-state ones on clusters 13.8 -> 3%, on one
-// CTA with runs of 2 and more columns 10.7 -> 4%; autoregulatory ones on clusters
-// 0.6 -> 0.3% (1.63 -> 1.18 times).  The others (one CTA of mRNA/protein or the
-// autoregulatory network, one column a thread of the two-state model, birth-death
-// models) gain on average and lose rarely, by at most a fifth, and keep the tile
-// kernel.
-// Measured: 152 thetas of 120 x 90, 13 times, 29.6 (tile) and 20.6 ms; 16 thetas
-// 5.3 and 20.5 ms; 1,000 thetas of 2 x 131 3.5 and 2.65 ms.
-bool tile_pays64(int kind, int64_t M, const TilePlan& tp, int nt, int G, int B, double overlap, int cluster, int threads,
-                 int64_t slab, size_t smem) {
-  const bool ts = kind == MJP_TWOSTATE, ar = kind == MJP_AUTOREG;
-  if (kind == MJP_BD1D || (double)B * tp.cluster <= kSms) return true;
-  if (tp.cluster == 1 && (!ts || tp.r == 1)) return true;
-  auto served = [](double ctas, int per, double latency, double work) {
-    const double n = std::ceil(ctas / kSms), full = std::floor(n / per), rest = n - full * per;
-    return full * std::max(latency, work * per) + (rest > 0.0 ? std::max(latency, work * rest) : 0.0);
+// Log-likelihoods of more CTAs than SMs: what counts is how much of an SM each
+// CTA takes, and there the tile kernel's halo pair rows (half of its work where a
+// CTA holds four), its cluster barriers, the warps it adds for the observation
+// groups and its 80 to 160 registers a thread can cost more than it saves against
+// stencil.cu, which holds 2 to 16 times the states per CTA in 64 registers.  Both
+// sides are estimated: an SM serves its CTAs in batches of as many as it holds,
+// and a batch takes the latency of a jump or the work of its CTAs.  Constants in
+// cycles, fitted to 8,000 calls (birth-death models of up to 30,000 states,
+// two-state ones of up to 950 columns, mRNA/protein boxes of up to 300 x 300,
+// autoregulatory ones of up to 120 x 200, 1 to 8,000 thetas, 1 to 100 times, up to
+// 6,000 groups); 80% of the estimates are within 30%.  Of the calls on clusters
+// the tile kernel was slower in (at worst, times), and is by this rule:
+// mRNA/protein FP64 15.6% (2.1) and 2% (1.3), two-state FP64 13.8% (2.0) and 3%
+// (1.3), autoregulatory FP32 28.7% (2.0) and 4% (1.4), FP64 0.6% (1.6) and 0.3%
+// (1.2), birth-death FP32 9% (2.9) and 3% (1.4); two-state FP64 on one CTA with
+// runs of 2 and more columns 10.7% (1.4) and 4% (1.2).  The shapes without an
+// entry gained on average and lost rarely, by at most a fifth.
+// Measured: 152 thetas of 120 x 90 mRNA/protein FP64, 13 times, 29.6 (tile) and
+// 20.6 ms, 16 thetas 5.3 and 20.5 ms; 1,606 thetas of the 38 x 148 autoregulatory
+// network FP32 131 and 64.6 ms; 1,000 thetas of 2 x 131 FP64 3.5 and 2.65 ms.
+bool tile_pays(int kind, int precision, int64_t M, const TilePlan& tp, int nt, int G, int B, double overlap, int cluster,
+               int threads, int64_t slab, size_t smem) {
+  struct Cost {
+    double lat, depth, work, group, group_lat;  // a jump; per pair and warp, in latency and work; per group step
+    double link;                                // tile: a hand-over or a cluster barrier
   };
+  struct Row {
+    int kind, precision;
+    bool clusters;
+    double margin;
+    Cost tile, shared;
+  };
+  static const Row rows[] = {
+      {MJP_MRNA_PROT2D, MJP_FP64, true, 1.15, {240, 158, 192, 39, 39, 1270}, {3110, 204, 292, 85, 208, 0}},
+      {MJP_TWOSTATE, MJP_FP64, true, 1.1, {820, 0, 138, 45, 45, 1160}, {1140, 112, 159, 66, 414, 0}},
+      {MJP_TWOSTATE, MJP_FP64, false, 1.05, {1640, 49, 121, 44, 44, 0}, {1140, 112, 159, 66, 414, 0}},
+      {MJP_AUTOREG, MJP_FP64, true, 1.05, {860, 181, 195, 42, 42, 554}, {1800, 344, 432, 68, 183, 0}},
+      {MJP_AUTOREG, MJP_FP32, true, 1.15, {830, 4.6, 22.5, 25.7, 25.7, 1560}, {2050, 14.6, 29.4, 38, 198, 0}},
+      {MJP_BD1D, MJP_FP32, true, 1.2, {1140, 0, 20.4, 21, 92, 0}, {1560, 12.3, 17.6, 32.6, 133, 0}},
+  };
+  if ((double)B * tp.cluster <= kSms || (tp.cluster == 1 && tp.r == 1)) return true;
+  const Row* row = nullptr;
+  for (const Row& r : rows)
+    if (r.kind == kind && r.precision == precision && r.clusters == (tp.cluster > 1)) row = &r;
+  if (!row) return true;
   // Warps that take a step of the active windows' groups, per jump: 32 groups
   // each, a window's last ones in a warp of their own.
   const double active = (double)G / nt * overlap;
   const double steps = std::min(active, active / 32.0 + 0.5 * std::max(1.0, overlap));
-  double work, lat;
-  // The tile kernel.
-  const double own = std::ceil(tp.geo.tx * tp.geo.ty / 32.0), ops = tp.r * (ts ? 7.0 : ar ? 13.0 : 10.0), depth = ops * std::ceil(own / 4.0);
-  double margin;
-  if (ar) {
-    margin = 1.05;
-    work = 15.0 * own * ops + 42.0 * steps;
-    lat = 860.0 + 55.7 * depth + 554.0 / tp.geo.period + 42.0 * steps / std::min(4.0, tp.threads / 32.0);
-  } else if (!ts) {
-    margin = 1.15;
-    work = 19.2 * own * ops + 39.0 * steps;
-    lat = 240.0 + 63.4 * depth + 1270.0 / tp.geo.period + 39.0 * steps / std::min(4.0, tp.threads / 32.0);
-  } else if (tp.cluster > 1) {
-    margin = 1.1;
-    work = 19.7 * own * ops + 45.0 * steps;
-    lat = 1980.0 + 45.0 * steps / std::min(4.0, tp.threads / 32.0);
+  auto served = [&](const Cost& c, int ctas, int per, double runs, double warps, double extra) {
+    // (The FP64 pipe takes a scheduler's warps one after the other.)
+    const double work = c.work * runs * warps + c.group * steps;
+    const double lat = c.lat + c.depth * runs * (precision == MJP_FP64 ? 4.0 * std::ceil(warps / 4.0) : warps) + extra;
+    per = std::max(1, std::min(per, 32));
+    const double n = std::ceil((double)B * ctas / kSms), full = std::floor(n / per), rest = n - full * per;
+    return full * std::max(lat, work * per) + (rest > 0.0 ? std::max(lat, work * rest) : 0.0);
+  };
+  const int regs = precision == MJP_FP64 ? (tp.r == 1 ? 96 : tp.r == 2 ? 128 : 160) : tp.r <= 2 ? 80 : 128;
+  const double tile = served(row->tile, tp.cluster, std::min(65536 / (tp.threads * regs), (int)(227 * 1024 / (tp.smem + 1024))),
+                             tp.r, std::ceil(tp.geo.tx * tp.geo.ty / 32.0),
+                             row->tile.link / (tp.geo.halo ? tp.geo.period : 1) +
+                                 row->tile.group_lat * steps / std::min(4.0, tp.threads / 32.0));
+  // stencil.cu: a thread walks a run of states (birth-death) or of pair rows of its
+  // column; from 8 states on one warp sums the observations.
+  double runs, warps;
+  if (kind == MJP_BD1D) {
+    runs = std::ceil((double)slab / (threads - 32));
+    warps = std::ceil(std::min<double>((double)slab, threads - 32) / 32.0);
   } else {
-    margin = 1.05;
-    work = 17.3 * own * ops + 44.0 * steps;
-    lat = 1640.0 + 28.0 * depth + 44.0 * steps / std::min(4.0, tp.threads / 32.0);
+    const double ty = std::max<double>(1.0, (double)((threads - 32) / M)), pair_rows = std::ceil(slab / (2.0 * M));
+    runs = std::ceil(pair_rows / ty);
+    warps = std::ceil(M * std::min(ty, pair_rows) / 32.0);
   }
-  const int regs = tp.r == 1 ? 96 : tp.r == 2 ? 128 : 160;
-  int per = std::min({65536 / (tp.threads * regs), (int)(227 * 1024 / (tp.smem + 1024)), 32});
-  const double tile = served((double)B * tp.cluster, std::max(1, per), lat, work);
-  // stencil.cu: a thread walks a run of pair rows of its column; from 4 of them on
-  // one warp sums the observations.
-  const double ty = std::max<double>(1.0, (double)((threads - 32) / M)), rows = std::ceil(slab / (2.0 * M)), runs = std::ceil(rows / ty);
-  const double warps = std::ceil(M * std::min(ty, rows) / 32.0), each = runs * (ts ? 7.0 : ar ? 17.0 : 12.0);
-  work = (ts ? 22.7 : ar ? 25.4 : 24.3) * warps * each + (ts ? 66.0 : ar ? 68.0 : 85.0) * steps;
-  lat = (ts ? 1140.0 : ar ? 1800.0 : 3110.0) + (ts ? 64.0 : ar ? 81.0 : 68.0) * each * std::ceil(warps / 4.0) +
-        (ts ? 414.0 : ar ? 183.0 : 208.0) * steps / (runs >= 4 ? 1.0 : threads / 32.0);
-  per = std::min({1024 / threads, (int)(227 * 1024 / (smem + 1024)), 32});
-  return margin * tile < served((double)B * cluster, std::max(1, per), lat, work);
+  const bool one_warp = (kind == MJP_BD1D ? runs : 2.0 * runs) >= 8.0;
+  const double shared = served(row->shared, cluster, std::min(1024 / threads, (int)(227 * 1024 / (smem + 1024))), runs, warps,
+                               row->shared.group_lat * steps / (one_warp ? 1.0 : threads / 32.0));
+  return row->margin * tile < shared;
 }
 
 cudaError_t launch_chain_tile(int kind, int precision, bool ll, const ChainParams& p, const TilePlan& tp,

@@ -93,10 +93,10 @@ __host__ __device__ constexpr int tile_jumps(size_t elt, int R) {
 // that hold a jump, on average (an estimate that only steers the choice).
 bool tile_plan(int kind, int precision, bool ll, int64_t M, int64_t P, int nt, int G, int maxmem, int B,
                double overlap, TilePlan* out);
-// Whether FP64 log-likelihoods of B thetas (any kind) take less time in this shape than in
+// Whether log-likelihoods of B thetas take less time in this shape than in
 // stencil.cu's (cluster, threads, states and shared memory of a CTA).
-bool tile_pays64(int kind, int64_t M, const TilePlan& tp, int nt, int G, int B, double overlap, int cluster, int threads,
-                 int64_t slab, size_t smem);
+bool tile_pays(int kind, int precision, int64_t M, const TilePlan& tp, int nt, int G, int B, double overlap, int cluster,
+               int threads, int64_t slab, size_t smem);
 cudaError_t launch_chain_tile(int kind, int precision, bool ll, const ChainParams& p, const TilePlan& tp,
                               cudaStream_t s);
 
