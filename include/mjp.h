@@ -104,7 +104,7 @@ extern "C" {
 #define MJP_OPT_ARENA 6         /* capacity (elements) of the planner's Poisson-weight store; 0 = automatic.  Windows
                                    that do not fit are generated in the chain by Algorithm 2's recurrence instead. */
 #define MJP_OPT_CHAIN 7         /* general CSR models: 0 or 1 = one launch per jump (default; nine state vectors of
-                                   scratch, two where nine take more than 16 GiB or cannot be allocated), 2 = the whole
+                                   scratch, two where nine do not pay or cannot be allocated), 2 = the whole
                                    chain in one cooperative launch with a bounded grid barrier per jump (two vectors;
                                    identical results; see MJP_OPT_WAIT_LIMIT).  Stencil models: 0 = automatic (the register-resident kernels for
                                    the log-likelihood of FP32 mRNA/protein boxes (automatic thread count or 256),

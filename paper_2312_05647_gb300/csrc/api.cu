@@ -67,6 +67,8 @@ struct mjp_model {
   DevBuf d_slice_ptr, d_slice_len, d_col, d_val, d_diag, d_perm;
   DevBuf d_bar;                            // grid barrier of the one-launch CSR chain
   bool csr_two = false;                    // the ring of vectors could not be allocated: two instead
+  int64_t csr_entries = 0;                 // with padding
+  bool csr_local = false;                  // most entries lie within kCsrNear states of the diagonal
   long long wait_limit = (long long)1 << 24;  // MJP_OPT_WAIT_LIMIT
   // workspace (scratch owned by the handle)
   DevBuf d_times, d_orig, d_win, d_info, d_theta, d_comp, d_status, d_ll;
@@ -198,7 +200,7 @@ double omega_bound(const mjp_model* m, const double* th) {
 // How many of the times' windows (about 16 sqrt(x) jumps each) hold a jump on
 // average, at the model's own theta; steers launch shapes only.
 double window_overlap(const mjp_model* m, const double* times, int nt) {
-  const double om = omega_bound(m, m->theta.data());
+  const double om = m->kind == MJP_CSR ? m->csr_omega : omega_bound(m, m->theta.data());
   double sum = 0.0, top = 1.0;
   for (int i = 0; i < nt; ++i) {
     const double x = om * times[i];
@@ -242,12 +244,29 @@ int arena_prepare(mjp_model* m, const double* host_theta, int B, const double* t
   return MJP_OK;
 }
 
+// Whether a ring of `ring` bytes costs the general-CSR chain more than the sums of
+// eight jumps at a time save.  The ring displaces the matrix (or itself) from the
+// L2, and adding a jump's vector to the outputs in the launch of the jump costs
+// little while few windows overlap.  Measured, two vectors against nine, 8 entries
+// a state, one and three times (overlap 1 and 2.9): FP64 random matrices of 300,000
+// states 1.1 times, of 500,000 0.91 and 0.96, of 2^20 0.95 and 0.97, of 2 million
+// 0.89 and 0.92, of 4 million 0.82 and 0.87 (with 12 times, overlap 10, 1.05 to
+// 1.13); band matrices of 2^20 states 1.04 and 1.13, of 2 million 0.92 and 1.00, of
+// 4 million 0.80 and 0.89.  FP32, bound by its gathers: random matrices of 4
+// million 1.01 and 1.07, of 8 million 0.95 and 1.01; band matrices 1.1 to 1.5.
+bool csr_ring_costs(const mjp_model* m, size_t ring, double overlap) {
+  const bool fp64 = m->precision == MJP_FP64;
+  const double mb = ((double)m->csr_entries * (fp64 ? 12 : 8) + (double)ring) / 1e6;
+  if (!fp64) return !m->csr_local && mb > 600.0 && overlap < 2.0;
+  return mb > (m->csr_local ? 180.0 : 64.0) && overlap < (m->csr_local ? 3.0 : 4.5);
+}
+
 // The general-CSR chain: planner (which also forms the weight table), windows
 // back to the host (the number of launches is the largest K), rho0 into the
 // in-degree order, then one launch per jump and one per kCsrBlock jumps for the
 // outputs (a ring of nine vectors), or one launch per jump that also adds its
-// vector to the outputs (two vectors: where nine take more than 16 GiB, and where
-// they cannot be allocated; 2^20 states FP32 34.7 instead of 32.6 ms).  Leaves the
+// vector to the outputs (two vectors: where nine take more than 16 GiB, where
+// they cannot be allocated, and where they cost more than they save).  Leaves the
 // outputs (times in ascending order, states in the internal order) in m->d_outp.
 int csr_run(mjp_model* m, const void* rho0, const double* sorted_times, int nt, int trunc_mode, double tol,
             cudaStream_t s, std::vector<Win>* wins) {
@@ -255,7 +274,9 @@ int csr_run(mjp_model* m, const void* rho0, const double* sorted_times, int nt, 
   const int64_t n = m->N;
   // The ring of vectors: a block of jumps and the one being formed.
   constexpr int kRingVecs = kCsrBlock + 1;
-  bool two = m->chain == 2 || m->csr_two || (size_t)kRingVecs * elt * n > ((size_t)16 << 30);
+  const size_t ring_bytes = (size_t)kRingVecs * elt * n;
+  bool two = m->chain == 2 || m->csr_two || ring_bytes > ((size_t)16 << 30) ||
+             csr_ring_costs(m, ring_bytes, window_overlap(m, sorted_times, nt));
   // Weights of a window: at most 20 sqrt(x) + 16 (x - 10 sqrt x .. x + 10 sqrt x + 10).
   double wcap = 2.0;
   // (Windows beyond the cap are refused below.)
@@ -272,7 +293,7 @@ int csr_run(mjp_model* m, const void* rho0, const double* sorted_times, int nt, 
         (rc = m->d_arena_ctl.ensure(16)) ||
         (m->precision == MJP_FP32 && (rc = m->d_comp.ensure(sizeof(float) * (size_t)nt * n))))
       return rc;
-    return m->d_rho2.ensure((size_t)(two ? 2 : kRingVecs) * elt * n);
+    return m->d_rho2.ensure(two ? 2 * elt * n : ring_bytes);
   };
   rc = allocate();
   if (rc == MJP_ERR_ALLOC && !two) {
@@ -509,11 +530,14 @@ int rate_model_create_csr(mjp_model** out, int64_t n, const int64_t* row_ptr, co
     int64_t s0 = q / 32, l = q % 32;
     for (int64_t j = 0; j < slen[s0]; ++j) ecol[sptr[s0] + j * 32 + l] = (int32_t)q;
   }
+  constexpr int64_t kCsrNear = 16384;
+  int64_t near = 0;
   std::vector<int32_t> fill(n, 0);
   for (int64_t i = 0; i < n; ++i)  // incoming entries in ascending source order
     for (int64_t j = row_ptr[i]; j < row_ptr[i + 1]; ++j) {
       const int64_t t = col[ord[j]];
       const int64_t q = perm[t], s0 = q / 32, l = q % 32;
+      near += std::abs(q - perm[i]) < kCsrNear ? 1 : 0;
       const int64_t slot = sptr[s0] + (int64_t)fill[t]++ * 32 + l;
       ecol[slot] = perm[i];
       eval[slot] = omega > 0.0 ? rate[ord[j]] / omega : 0.0;
@@ -527,6 +551,9 @@ int rate_model_create_csr(mjp_model** out, int64_t n, const int64_t* row_ptr, co
   m->N = n; m->M = n; m->P = 1;
   m->csr_omega = omega;
   m->nslices = nslices;
+  m->csr_entries = npad;
+  m->csr_local = 2 * near >= row_ptr[n];
+  m->csr_local = 2 * near >= row_ptr[n];
   const size_t elt = precision == MJP_FP64 ? 8 : 4;
   int rc = 0;
   if ((rc = m->d_slice_ptr.ensure(sizeof(int64_t) * nslices)) || (rc = m->d_slice_len.ensure(sizeof(int32_t) * nslices)) ||

@@ -23,8 +23,8 @@
 // step per jump), instead of every jump reading and writing every active
 // output.
 //
-// Where only two vectors are held (more than 16 GiB for nine, or no memory for
-// them), the launch of a jump adds the vector it reads to the active outputs.
+// Where only two vectors are held (api.cu: no memory for nine, or a ring that does
+// not pay), the launch of a jump adds the vector it reads to the active outputs.
 //
 // Alternative (MJP_OPT_CHAIN = 2): the whole chain in one cooperative launch
 // (all CTAs co-resident), the outputs accumulated at every jump, jumps

@@ -45,3 +45,36 @@ def test_same_bits(n, degrees, prec):
         two = _run_two(rp, col, val, prec, rho0, times, **kw)
         assert np.array_equal(two, _run(rp, col, val, prec, rho0, times, 0, **kw))
         assert np.array_equal(two, _run(rp, col, val, prec, rho0, times, 2, **kw))
+
+
+def test_a_ring_that_leaves_the_l2_is_not_taken():
+    """3 million states, random FP64 entries, one time: nine vectors took 1.2 times as long as two."""
+    import torch
+    import paper_2312_05647_gb300 as mjp
+    n, d = 3000000, 4
+    gen = np.random.default_rng(5)
+    off = np.sort(gen.integers(0, n // d - 1, (n, d)) + np.arange(d) * (n // d), axis=1) + 1
+    col = np.sort((np.arange(n)[:, None] + off) % n, axis=1).ravel().astype(np.int32)
+    rp, val = np.arange(n + 1, dtype=np.int64) * d, gen.lognormal(0.0, 1.0, n * d)
+    rho0 = torch.full((n,), 1.0 / n, dtype=torch.float64, device="cuda")
+    f = getattr(mjp.capi.lib(), "_ZN3mjp13model_csr_twoEP9mjp_model")
+    f.restype, f.argtypes = None, [ctypes.c_void_p]
+    ms, outs = [], []
+    for two in (False, True):
+        m = mjp.Model.from_csr(n, rp, col, val, 2)
+        if two:
+            f(m._h)
+        om = m.expv(rho0, [1e-9], info=True)[1]["omega"]
+        best = np.inf
+        for _ in range(4):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            torch.cuda.synchronize()
+            a.record()
+            out = m.expv(rho0, [60.0 / om])
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b))
+        ms.append(best)
+        outs.append(out)
+    assert torch.equal(outs[0], outs[1])
+    assert ms[0] <= 1.05 * ms[1], ms
