@@ -841,7 +841,7 @@ int expv_series(mjp_model* m, const void* rho0, const double* times, int ntimes,
   bool use_reg1 = false;
   SmallPlan sp = {};
   const bool automatic = m->chain == 0 && m->cluster == 0 && m->threads == 0 && m->kcap <= (1 << 30) - 1;
-  const double overlap = automatic ? window_overlap(m, st.data(), nt) : 0.0;
+  const double overlap = window_overlap(m, st.data(), nt);
   const bool use_small = automatic && chain_small_plan(m->kind, m->precision, m->M, m->N, nt, overlap, &sp);
   if (!use_small && m->kind == MJP_BD1D && m->chain != 1 && m->threads == 0) {
     const int c0 = m->cluster > 0 ? m->cluster : 1, c1 = m->cluster > 0 ? m->cluster : 8;
@@ -890,7 +890,11 @@ int expv_series(mjp_model* m, const void* rho0, const double* times, int ntimes,
   cp.renorm = (m->precision == MJP_FP32) ? m->renorm : 0;
   cp.slab = slab; cp.status = pp.status; cp.wait_limit = m->wait_limit;
   if (use_small) MJP_CUDA(launch_chain_small(m->kind, m->precision, cp, sp, s));
-  else if (use_reg1) MJP_CUDA(launch_chain_reg1d(m->precision, cp, rp1, s));
+  // Sums of a round's only window in registers: they cost the FP32 kernel 36
+  // spilled bytes, up to 18% of a call whose windows overlap by more (two to 200
+  // times, 500 to 30,000 states), and save 7 to 60% below; FP64, which spills
+  // nothing, 0 to 26% at every overlap.
+  else if (use_reg1) MJP_CUDA(launch_chain_reg1d(m->precision, cp, rp1, m->precision == MJP_FP64 || overlap <= 1.1, s));
   else if (use_tile) MJP_CUDA(launch_chain_tile(m->kind, m->precision, false, cp, xp, s));
   else MJP_CUDA(launch_chain_stencil(m->kind, m->precision, 0, cp, C, T, s));
   if ((rc = mark(m, 2, s))) return rc;

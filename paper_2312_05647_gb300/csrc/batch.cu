@@ -209,7 +209,7 @@ int regroup_reg(mjp_batch* b, int halo) {
     g.smem = g.rp.smem;
     ChainParams prep = {};  // set kernel attributes now (never inside graph capture)
     prep.B = 0;
-    MJP_CUDA(launch_chain_reg1d(b->precision, prep, g.rp, nullptr));
+    MJP_CUDA(launch_chain_reg1d(b->precision, prep, g.rp, true, nullptr));
     int rc = g.d_map.ensure(sizeof(int32_t) * g.jobs.size());
     if (rc) return rc;
     MJP_CUDA(cudaMemcpy(g.d_map.p, g.jobs.data(), sizeof(int32_t) * g.jobs.size(), cudaMemcpyHostToDevice));
@@ -294,7 +294,7 @@ int enqueue(mjp_batch* b, void* out, cudaStream_t s) {
     cp.renorm = b->precision == MJP_FP32 ? b->renorm : 0; cp.slab = 1; cp.status = pp.status;
     cp.jobN = pp.jobN; cp.job_off = b->d_off.as<int64_t>(); cp.job_map = g.d_map.as<int32_t>();
     cp.job_s0 = b->d_s0.as<int64_t>(); cp.tile_max = g.tile; cp.arena = b->d_arena.p;
-    if (g.reg) MJP_CUDA(launch_chain_reg1d(b->precision, cp, g.rp, b->side[gi]));
+    if (g.reg) MJP_CUDA(launch_chain_reg1d(b->precision, cp, g.rp, true, b->side[gi]));
     else MJP_CUDA(launch_chain_stencil(MJP_BD1D, b->precision, 0, cp, g.cluster, g.threads, b->side[gi]));
     MJP_CUDA(cudaEventRecord(b->ev_join[gi], b->side[gi]));
     MJP_CUDA(cudaStreamWaitEvent(s, b->ev_join[gi], 0));

@@ -237,7 +237,8 @@ struct Reg1dPlan {
 bool chain_reg1d_plan(int precision, int64_t Nmax, int ntimes, int cluster, int halo, Reg1dPlan* out,
                       bool small = false);
 int64_t chain_reg1d_max_states(int precision);
-cudaError_t launch_chain_reg1d(int precision, const ChainParams& p, const Reg1dPlan& rp, cudaStream_t s);
+// one: windows seldom overlap (always, for a single time).
+cudaError_t launch_chain_reg1d(int precision, const ChainParams& p, const Reg1dPlan& rp, bool one, cudaStream_t s);
 // Register-resident two-state chain (stencil_regts.cu): FP32 loglik, one CTA
 // per theta, groups of at most two members.
 struct RegTsPlan {

@@ -104,7 +104,9 @@ struct RotSeq<P1, O, 0> {
   __device__ __forceinline__ static void run(F&) {}
 };
 
-template <typename T, int QP, int kMaxT>
+// ONE: rounds that meet one window at most keep its sums in registers (round_one
+// below).
+template <typename T, int QP, int kMaxT, bool ONE>
 __global__ void __launch_bounds__(kMaxT, 1) chain_reg1d_kernel(const ChainParams p, const int halo) {
   using T2 = typename Pair<T>::type;
   constexpr int R = 2 * QP;       // states per lane
@@ -638,16 +640,19 @@ __global__ void __launch_bounds__(kMaxT, 1) chain_reg1d_kernel(const ChainParams
   advance(kE, lo, hi);
   if (wact) accumulate(kE, lo, hi, std::integral_constant<int, 0>{});
   while (k <= Kmax) {
-    while (lo < nt && t_K[lo] < k) ++lo;
-    int h1 = hi;
-    while (h1 + 1 < nt && t_L[h1 + 1] < k + P1) ++h1;
-    if (h1 <= lo) {
-      hi = h1;
-      if (wact) round_one(h1 == lo ? lo : -1);
-      else k = min(k + P1, Kmax + 1);
-    } else {
-      RotSeq<P1, 0, P1>::run(jump_acc);
+    bool one = false;
+    if constexpr (ONE) {
+      while (lo < nt && t_K[lo] < k) ++lo;
+      int h1 = hi;
+      while (h1 + 1 < nt && t_L[h1 + 1] < k + P1) ++h1;
+      one = h1 <= lo;
+      if (one) {
+        hi = h1;
+        if (wact) round_one(h1 == lo ? lo : -1);
+        else k = min(k + P1, Kmax + 1);
+      }
     }
+    if (!one) RotSeq<P1, 0, P1>::run(jump_acc);
     const int k_e = k - 1;
     if (k_e >= Kmax) break;
     defect();
@@ -661,11 +666,11 @@ __global__ void __launch_bounds__(kMaxT, 1) chain_reg1d_kernel(const ChainParams
   cp_async_wait<0>();
 }
 
-template <typename T, int QP, int kMaxT>
+template <typename T, int QP, int kMaxT, bool ONE>
 cudaError_t launch_reg1d_typed(const ChainParams& p, const Reg1dPlan& rp, cudaStream_t s) {
   static int smem_set = 0;
   static bool nonportable = false;
-  auto kern = chain_reg1d_kernel<T, QP, kMaxT>;
+  auto kern = chain_reg1d_kernel<T, QP, kMaxT, ONE>;
   cudaError_t e;
   if ((int)rp.smem > smem_set) {
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rp.smem);
@@ -741,12 +746,17 @@ int64_t chain_reg1d_max_states(int precision) {
   return (int64_t)(maxt / 32) * (60 * qp);  // warp windows overlap by two lanes' runs
 }
 
-cudaError_t launch_chain_reg1d(int precision, const ChainParams& p, const Reg1dPlan& rp, cudaStream_t s) {
+template <bool ONE>
+static cudaError_t launch_reg1d(int precision, const ChainParams& p, const Reg1dPlan& rp, cudaStream_t s) {
   if (rp.qp == kQPSmall)
-    return precision == MJP_FP64 ? launch_reg1d_typed<double, kQPSmall, kMaxTSmall>(p, rp, s)
-                                 : launch_reg1d_typed<float, kQPSmall, kMaxTSmall>(p, rp, s);
-  if (precision == MJP_FP64) return launch_reg1d_typed<double, kQP64, kMaxT64>(p, rp, s);
-  return launch_reg1d_typed<float, kQP32, kMaxT32>(p, rp, s);
+    return precision == MJP_FP64 ? launch_reg1d_typed<double, kQPSmall, kMaxTSmall, ONE>(p, rp, s)
+                                 : launch_reg1d_typed<float, kQPSmall, kMaxTSmall, ONE>(p, rp, s);
+  if (precision == MJP_FP64) return launch_reg1d_typed<double, kQP64, kMaxT64, ONE>(p, rp, s);
+  return launch_reg1d_typed<float, kQP32, kMaxT32, ONE>(p, rp, s);
+}
+
+cudaError_t launch_chain_reg1d(int precision, const ChainParams& p, const Reg1dPlan& rp, bool one, cudaStream_t s) {
+  return one ? launch_reg1d<true>(precision, p, rp, s) : launch_reg1d<false>(precision, p, rp, s);
 }
 
 }  // namespace mjp
