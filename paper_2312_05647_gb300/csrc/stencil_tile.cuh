@@ -48,9 +48,15 @@
 //
 // Bound: instruction issue and the latency of a jump (reads behind a barrier,
 // the dependent multiply-adds) in FP32, the FP64 pipe (64 cycles per warp
-// instruction and scheduler) in FP64; DRAM and L2 are idle.  Spills must not
-// happen here: with the shared memory this full they miss the L1 and cost an
-// L2 access each (a version with 90 spilled bytes ran four times slower).
+// instruction and scheduler) in FP64; DRAM and L2 are idle (the autoregulatory
+// instance below: issue slots 44% busy, L2 0.1%).  Spills: an early version with 90
+// bytes spilled inside the jump and nearly all of the shared memory taken ran four
+// times slower, its accesses missing the small L1 left.  The thread bounds leave
+// some instances with spills all the same (-Xptxas -v, bytes stored): FP32
+// log-likelihoods 4 to 16 with R = 1, 8 to 120 with R = 2, 16 with R = 4 on clusters,
+// birth-death R = 8 64, autoregulatory R = 10 160 (the 40 x 120 case); FP32 transient
+// distributions on clusters 4 (R = 3) to 88 (R = 4); FP64 4.  Theirs stay in the L1
+// (the same 0.1% of the L2).
 // Measured against the shared-memory kernel (one GB300): autoregulatory
 // network 40 x 120, 152 thetas, 50 times, FP32 12.5 -> 2.0 ms; birth-death N =
 // 64, 10^4 thetas, FP64 7.61 -> 3.55 ms; two-state N_R = 131, one theta, FP64
