@@ -1180,7 +1180,9 @@ int loglik(mjp_model* m, const mjp_obs* obs, const double* theta, int B, double*
   bool use_tile = !use_reg && !use_ts && m->chain == 0 && m->cluster == 0 && m->threads == 0 &&
                   m->kcap <= (1 << 30) - 1 &&
                   tile_plan(m->kind, m->precision, true, m->M, m->P, nt, obs->G, obs->maxmem, B, overlap, &xp);
-  if (use_tile && B > 1 && stencil_config(m, 1, nt, obs->G, nmem_list, &C, &T, &slab) == MJP_OK)
+  // (Asked only where tile_pays looks at the other side.)
+  if (use_tile && (double)B * xp.cluster > 152.0 && (xp.cluster > 1 || xp.r > 1) &&
+      stencil_config(m, 1, nt, obs->G, nmem_list, &C, &T, &slab) == MJP_OK)
     use_tile = tile_pays(m->kind, m->precision, m->M, xp, nt, obs->G, B, overlap, C, T, slab,
                          chain_stencil_smem(m->kind, m->precision, 1, m->M, m->P, slab, nt, obs->G, nmem_list));
   if (!use_reg && !use_ts && !use_tile && (rc = stencil_config(m, 1, nt, obs->G, nmem_list, &C, &T, &slab))) return rc;
